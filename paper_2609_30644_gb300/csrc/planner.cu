@@ -555,6 +555,15 @@ __device__ __forceinline__ void bfs_connected(const int *adj, const int *deg, in
     if (threadIdx.x == 0) *connected = n > 1 && level[1] >= 0;
 }
 
+// Shared memory of link_body: the checked edges of 64 gathered vertices (their
+// neighbour, or -1), the degrees of the roadmap's vertices and the BFS bitmaps.
+constexpr int kLinkVerts = 16384;
+struct LinkShared {
+    int es[64 * kKmax];
+    uint8_t deg[kLinkVerts];
+    unsigned vis[kLinkVerts / 32], fr[kLinkVerts / 32], nx[kLinkVerts / 32];
+};
+
 // ---------------------------------------------------------------------------
 // batched ROADMAP rounds: one job per robot of every problem that needs a
 // round; every kernel takes a job dimension (blockIdx.y), so a round costs a
@@ -686,14 +695,112 @@ __global__ void k_rmb_edges(const RmJob *__restrict__ jobs) {
     rmb_edges_body(jobs[blockIdx.y], blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-__global__ void k_rmb_link(const RmJob *__restrict__ jobs) {
-    const RmJob &J = jobs[blockIdx.y];
-    link_edges(J.evalid, J.ea, J.eb, J.m * kKmax, J.adj, J.deg);
+// The last phase of a robot's round, in one block: links the checked edges and
+// decides whether vertex 1 (the goal) can be reached from vertex 0 (the start).
+//
+// The lists come out as link_edges builds them.  A gathered vertex j owns the
+// kKmax consecutive edge slots of its own neighbour list, all of them to lower
+// indices, so its own appends precede every append to it by a later vertex:
+// one warp per gathered vertex ranks its list with two ballots, then one warp
+// walks the gathered vertices in order and appends each to its neighbours'
+// lists (distinct vertices, so the 64 slots go side by side).  Bound by
+// latency, not by bytes: the edges and degrees are staged in shared memory, so
+// a step of that walk is a shared load, compare and store.  Links are never
+// removed, so a connected roadmap stays connected and is not searched again;
+// the search keeps its visited set and frontier as shared bitmaps and reads a
+// frontier vertex's list 16 bytes at a time.  Measured per round (8 arms,
+// up to 1,500 vertices): 132 us with link_edges and bfs_connected, whose every
+// step waits on global memory, 28 us here.  Roadmaps above kLinkVerts
+// vertices (the shared tables' room) keep the global-memory form.
+__device__ __forceinline__ void link_body(const RmJob &J, LinkShared &sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int n = *J.count, m = J.m, first = J.first;
+    const bool was_connected = J.n_old > 2 && *J.conn != 0;
+    int *adj = J.adj, *deg = J.deg;
+    __syncthreads();  // every thread has read *J.conn before it is rewritten
+    if (n > kLinkVerts) {
+        if (tid < 32) link_edges(J.evalid, J.ea, J.eb, m * kKmax, adj, deg);
+        __syncthreads();
+        bfs_connected(adj, deg, n, J.level, J.conn);
+        return;
+    }
+    for (int v = tid; v < n; v += blockDim.x) sh.deg[v] = (uint8_t)min(deg[v], kKmax);
+    for (int j0 = 0; j0 < m; j0 += 64) {
+        __syncthreads();
+        for (int i = tid; i < 64 * kKmax; i += blockDim.x) {
+            const int e = j0 * kKmax + i;
+            sh.es[i] = e < m * kKmax && J.evalid[e] && J.ea[e] >= 0 ? J.eb[e] : -1;
+        }
+        __syncthreads();
+        const int jn = min(64, m - j0);
+        for (int j = warp; j < jn; j += nwarps) {
+            const int x = first + j0 + j, d0 = sh.deg[x];
+            const int y0 = sh.es[j * kKmax + lane], y1 = sh.es[j * kKmax + 32 + lane];
+            const unsigned b0 = __ballot_sync(0xffffffffu, y0 >= 0);
+            const unsigned b1 = __ballot_sync(0xffffffffu, y1 >= 0);
+            const unsigned below = (1u << lane) - 1u;
+            const int p0 = d0 + __popc(b0 & below), p1 = d0 + __popc(b0) + __popc(b1 & below);
+            if (y0 >= 0 && p0 < kKmax) adj[(size_t)x * kKmax + p0] = y0;
+            if (y1 >= 0 && p1 < kKmax) adj[(size_t)x * kKmax + p1] = y1;
+            if (lane == 0) sh.deg[x] = (uint8_t)min(d0 + __popc(b0) + __popc(b1), kKmax);
+        }
+        __syncthreads();
+        if (warp == 0)
+            for (int j = 0; j < jn; ++j) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int y = sh.es[j * kKmax + 32 * h + lane];
+                    if (y < 0) continue;
+                    const int d = sh.deg[y];
+                    if (d >= kKmax) continue;
+                    adj[(size_t)y * kKmax + d] = first + j0 + j;
+                    sh.deg[y] = (uint8_t)(d + 1);
+                }
+                __syncwarp();  // the next vertex reads these degrees
+            }
+    }
+    __syncthreads();
+    for (int v = tid; v < n; v += blockDim.x) deg[v] = sh.deg[v];
+    if (was_connected) return;
+    const int words = (n + 31) >> 5;
+    for (int w = tid; w < words; w += blockDim.x) {
+        sh.vis[w] = sh.fr[w] = w == 0 ? 1u : 0u;
+        sh.nx[w] = 0u;
+    }
+    __syncthreads();
+    for (;;) {  // one level each; every level but the last adds a vertex
+        for (int v = tid; v < n; v += blockDim.x) {
+            if (!((sh.fr[v >> 5] >> (v & 31)) & 1u)) continue;
+            const int dg = sh.deg[v];
+            const int4 *row = reinterpret_cast<const int4 *>(adj + (size_t)v * kKmax);
+#pragma unroll 4
+            for (int k = 0; k < dg; k += 4) {
+                const int4 y = row[k >> 2];
+                const int ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (k + u < dg && ys[u] >= 0 && ys[u] < n &&
+                        !((sh.vis[ys[u] >> 5] >> (ys[u] & 31)) & 1u))
+                        atomicOr(&sh.nx[ys[u] >> 5], 1u << (ys[u] & 31));
+            }
+        }
+        __syncthreads();
+        bool more = false;
+        for (int w = tid; w < words; w += blockDim.x) {
+            const unsigned f = sh.nx[w] & ~sh.vis[w];
+            sh.fr[w] = f;
+            sh.vis[w] |= f;
+            sh.nx[w] = 0u;
+            more |= f != 0u;
+        }
+        if (!__syncthreads_or(more) || (n > 1 && (sh.vis[0] >> 1) & 1u)) break;
+    }
+    if (tid == 0) *J.conn = n > 1 && ((sh.vis[0] >> 1) & 1u) != 0u;
 }
 
-__global__ void __launch_bounds__(1024) k_rmb_bfs(const RmJob *__restrict__ jobs) {
-    const RmJob &J = jobs[blockIdx.y];
-    bfs_connected(J.adj, J.deg, *J.count, J.level, J.conn);
+__global__ void __launch_bounds__(256) k_rmb_link(const RmJob *__restrict__ jobs) {
+    __shared__ LinkShared sh;
+    link_body(jobs[blockIdx.y], sh);
 }
 
 // (vertex count, connected) of every job, for one copy to the host.
@@ -975,6 +1082,7 @@ static mrpop_status planner_init(mrpop_problem *p, Planner **out) {
         PL_TRY(dalloc(&r.eb, (size_t)E + 2 * kKmax));
         PL_TRY(dalloc(&r.level, (size_t)rcap));
         PL_TRY(dalloc(&r.d_conn, 1));
+        PL_TRY(cudaMemset(r.d_conn, 0, sizeof(int)));
         // vertices 0 and 1: the robot's start and goal
         for (int d = 0; d < dof; ++d) {
             PL_TRY(cudaMemcpy(r.q + (size_t)d * rcap, &p->start[qoff + d], sizeof(float),
@@ -1195,8 +1303,7 @@ static mrpop_status roadmap_round_jobs(const std::vector<Planner *> &pls, cudaSt
     k_rmb_edges<<<dim3((e_max + 127) / 128, nj), 128, 0, st>>>(d_jobs);
     PL_TRY(cudaGetLastError());
     ST_TRY(launch_validate_batch(d_vp + nj, nj, spl_e, w_e, b_e, s_e, false, st));
-    k_rmb_link<<<dim3(1, nj), 32, 0, st>>>(d_jobs);
-    k_rmb_bfs<<<dim3(1, nj), 1024, 0, st>>>(d_jobs);
+    k_rmb_link<<<dim3(1, nj), 256, 0, st>>>(d_jobs);
     k_rmb_collect<<<(nj + 127) / 128, 128, 0, st>>>(d_jobs, nj, d_out);
     PL_TRY(cudaGetLastError());
     std::vector<int> out(2 * (size_t)nj);
@@ -1613,13 +1720,16 @@ static mrpop_status plan_batch(mrpop_problem *const *ps, int n, double budget, i
 // Alg. 1 for every problem of the batch until each is done (time budget,
 // step budget or target cost).  Every problem carries a state machine of
 // phases -- a ROADMAP round is sample, candidate validation, append,
-// NEIGHBORS, candidate edges, edge validation and link + BFS for each robot
-// in turn; a search step is the nine phases of the stepped form; an
+// NEIGHBORS, candidate edges, edge validation and link + BFS, each phase over
+// all of the problem's robots at once (their roadmaps and random streams are
+// independent, and a round is a chain of short phases, K times as long robot
+// by robot: twelve problems of 2-8 arms, 24 steps, 77 ms of kernel time robot
+// by robot and 62 ms with the phases over all robots and link_body); a search step is the nine phases of the stepped form; an
 // incumbent candidate is re-checked at a quarter of the resolution -- and
 // each phase is cut into chunks (256 samples or iterations, 16 NEAREST
 // queries, 32 edges, 8 NEIGHBORS queries).  CTAs claim chunks of any problem
 // with one atomic add on the problem's phase word, which carries the phase
-// itself (kind, robot, chunk count) beside the next chunk, so a claim always
+// itself (kind, chunk count) beside the next chunk, so a claim always
 // names the phase it belongs to.  The CTA that finishes a phase's last chunk
 // runs the transition (Alg. 1 bookkeeping on the device, in the stepped
 // form's order) and publishes the next phase.  No CTA waits for another: a
@@ -1638,15 +1748,15 @@ enum PKind : int {
 constexpr int kPerThreads = 256;          // threads per persistent CTA (= kStepIters)
 constexpr int kPerWarps = kPerThreads / 32;
 constexpr int kPerEdges = 32;             // edges per validation chunk
+constexpr int kPerConfigs = 8;            // roadmap candidates per validation chunk (a warp each)
 constexpr int kFineCap = 16384;           // sub-edges per fine re-check window
 constexpr int kTraceCap = 256;            // incumbents recorded per problem
 constexpr int kHistCap = 64;              // incumbent paths kept per problem
 static_assert(kPerThreads == kStepIters, "one search-step iteration per thread");
 
-// Phase word: kind (6 bits) | robot (6) | chunk count (20) | next chunk (32).
-__host__ __device__ __forceinline__ unsigned long long phase_word(int kind, int robot, int total) {
-    return ((unsigned long long)kind << 58) | ((unsigned long long)(robot & 63) << 52) |
-           ((unsigned long long)(total & 0xFFFFF) << 32);
+// Phase word: kind (6 bits) | unused (6) | chunk count (20) | next chunk (32).
+__host__ __device__ __forceinline__ unsigned long long phase_word(int kind, int total) {
+    return ((unsigned long long)kind << 58) | ((unsigned long long)(total & 0xFFFFF) << 32);
 }
 
 struct PState {
@@ -1706,11 +1816,11 @@ __device__ __forceinline__ unsigned long long gtimer() {
 
 __device__ __forceinline__ int chunks_of(int n, int per) { return n <= 0 ? 0 : (n + per - 1) / per; }
 
-// Validation of edges [chunk * 32, chunk * 32 + 32) of vp (count edges in all).
-__device__ __noinline__ void val_chunk(const VParams &vp, int chunk, int count, float4 *sm4,
-                                       int *s_next) {
+// Validation of edges [chunk * per, chunk * per + per) of vp (count edges in all).
+__device__ __noinline__ void val_chunk(const VParams &vp, int chunk, int per, int count,
+                                       float4 *sm4, int *s_next) {
     if (threadIdx.x == 0) *s_next = 0;
-    const int e0 = chunk * kPerEdges, e1 = min(count, e0 + kPerEdges);
+    const int e0 = chunk * per, e1 = min(count, e0 + per);
     vb::validate_body<vb::kVerdict, false, true>(vp, sm4, e0, e1, s_next);
     __syncthreads();
 }
@@ -1847,13 +1957,33 @@ __device__ void fine_accept(PState &ps) {
     }
 }
 
-__device__ void run_chunk(PState &ps, int kind, int r, int c, float4 *sm4, NnShared<kPerThreads> &nn,
+// Chunks of one robot in a ROADMAP phase (the same for every robot of a
+// problem: the chunk's body skips what lies beyond its robot's own counts).
+__device__ __forceinline__ int rm_chunks(const PState &ps, int kind) {
+    const RmJob &J = ps.jobs[0];
+    switch (kind) {
+        case PK_RM_SAMPLE: return chunks_of(J.nc, kPerThreads);
+        case PK_RM_VALC: return chunks_of(J.nc, kPerConfigs);
+        case PK_RM_NB: return chunks_of(ps.n_per_round + 2, kPerWarps);
+        case PK_RM_EDGES: return chunks_of(J.emax, kPerThreads);
+        case PK_RM_VALE: return chunks_of(J.emax, kPerEdges);
+        default: return 1;
+    }
+}
+
+__device__ void run_chunk(PState &ps, int kind, int c, float4 *sm4, NnShared<kPerThreads> &nn,
                           int *wsum, int *s_next, double *red) {
     const Slot &S = *ps.slot;
     const int tid = threadIdx.x;
+    int r = 0;
+    if (kind >= PK_RM_SAMPLE && kind <= PK_RM_LINK) {  // chunk c of all robots' chunks
+        const int per = rm_chunks(ps, kind);
+        r = c / per;
+        c -= r * per;
+    }
     switch (kind) {
         case PK_RM_SAMPLE: rmb_sample_body(ps.jobs[r], c * kPerThreads + tid); break;
-        case PK_RM_VALC: val_chunk(ps.vp[3 + r], c, ps.jobs[r].nc, sm4, s_next); break;
+        case PK_RM_VALC: val_chunk(ps.vp[3 + r], c, kPerConfigs, ps.jobs[r].nc, sm4, s_next); break;
         case PK_RM_APPEND: {
             RmJob &J = ps.jobs[r];
             append_valid(J.cand, J.cvalid, J.nc, J.dof, J.want, J.q, J.rcap, J.count);
@@ -1866,27 +1996,24 @@ __device__ void run_chunk(PState &ps, int kind, int r, int c, float4 *sm4, NnSha
         }
         case PK_RM_NB: rmb_neighbors_body(ps.jobs[r], c * kPerWarps + (tid >> 5)); break;
         case PK_RM_EDGES: rmb_edges_body(ps.jobs[r], c * kPerThreads + tid); break;
-        case PK_RM_VALE: val_chunk(ps.vp[3 + ps.K + r], c, ps.jobs[r].emax, sm4, s_next); break;
+        case PK_RM_VALE: val_chunk(ps.vp[3 + ps.K + r], c, kPerEdges, ps.jobs[r].emax, sm4, s_next); break;
         case PK_RM_LINK: {
-            const RmJob &J = ps.jobs[r];
-            if (tid < 32) link_edges(J.evalid, J.ea, J.eb, J.m * kKmax, J.adj, J.deg);
-            __syncthreads();
-            bfs_connected(J.adj, J.deg, *J.count, J.level, J.conn);
+            link_body(ps.jobs[r], *reinterpret_cast<LinkShared *>(sm4));
             break;
         }
         case PK_ST_SAMPLE: sample_body(S, tid); break;
         case PK_ST_NN0: nearest_body<0, kPerThreads>(S, c, nn); break;
         case PK_ST_ORACLE: oracle_body(S, tid); break;
-        case PK_ST_VAL1: val_chunk(ps.vp[0], c, kStepIters, sm4, s_next); break;
+        case PK_ST_VAL1: val_chunk(ps.vp[0], c, kPerEdges, kStepIters, sm4, s_next); break;
         case PK_ST_INSERT: insert_body(S, wsum); break;
         case PK_ST_NN1: nearest_body<1, kPerThreads>(S, c, nn); break;
         case PK_ST_CONN: conn_prep_body(S, tid); break;
-        case PK_ST_VAL2: val_chunk(ps.vp[1], c, kStepIters, sm4, s_next); break;
+        case PK_ST_VAL2: val_chunk(ps.vp[1], c, kPerEdges, kStepIters, sm4, s_next); break;
         case PK_ST_SOLUTION:
             solution_body(S, tid);
             solution_candidate(ps, red);
             break;
-        case PK_FINE_VAL: val_chunk(ps.vp[2], c, ps.fine_cnt, sm4, s_next); break;
+        case PK_FINE_VAL: val_chunk(ps.vp[2], c, kPerEdges, ps.fine_cnt, sm4, s_next); break;
         case PK_FINE_ACCEPT: fine_accept(ps); break;
         default: break;
     }
@@ -1899,13 +2026,21 @@ struct PDecision {
     int reset;
 };
 
-__device__ unsigned long long round_setup(PState &ps, int k) {
-    RmJob &J = ps.jobs[k];
-    const int n = *J.count;
-    J.ctr = (unsigned long long)(ps.step + 1) * 0x100000ull + (unsigned long long)n * 4096ull;
-    J.want = n >= ps.rcap ? 0 : min(ps.n_per_round, ps.rcap - n);
-    J.n_old = n;
-    return phase_word(PK_RM_SAMPLE, k, chunks_of(J.nc, kPerThreads));
+// Phase word of a ROADMAP phase over every robot.  The chunk count fits its 20
+// bits: at most 16 robots of (4,096 + 2) * 64 / 32 edge chunks.
+__device__ __forceinline__ unsigned long long rm_word(const PState &ps, int kind) {
+    return phase_word(kind, ps.K * rm_chunks(ps, kind));
+}
+
+__device__ unsigned long long round_setup(PState &ps) {
+    for (int k = 0; k < ps.K; ++k) {
+        RmJob &J = ps.jobs[k];
+        const int n = *J.count;
+        J.ctr = (unsigned long long)(ps.step + 1) * 0x100000ull + (unsigned long long)n * 4096ull;
+        J.want = n >= ps.rcap ? 0 : min(ps.n_per_round, ps.rcap - n);
+        J.n_old = n;
+    }
+    return rm_word(ps, PK_RM_SAMPLE);
 }
 
 __device__ unsigned long long start_step(PState &ps) {
@@ -1918,7 +2053,7 @@ __device__ unsigned long long start_step(PState &ps) {
     C.best_key = ~0ull;
     C.overflow = 0;
     if (C.mode == 2) return 0ull;  // an idle step changes nothing: the outer iteration ends
-    return phase_word(PK_ST_SAMPLE, 0, 1);
+    return phase_word(PK_ST_SAMPLE, 1);
 }
 
 __device__ PDecision begin_outer(PState &ps, unsigned long long now, unsigned long long deadline);
@@ -1929,7 +2064,7 @@ __device__ PDecision end_outer(PState &ps, unsigned long long now, unsigned long
 }
 
 __device__ PDecision begin_outer(PState &ps, unsigned long long now, unsigned long long deadline) {
-    PDecision d{phase_word(PK_DONE, 0, 0), 0};
+    PDecision d{phase_word(PK_DONE, 0), 0};
     if (!ps.active) return d;
     if (now >= deadline) {
         ps.timed_out = 1;
@@ -1937,7 +2072,7 @@ __device__ PDecision begin_outer(PState &ps, unsigned long long now, unsigned lo
     }
     if (ps.max_steps > 0 && ps.steps_done >= ps.max_steps) return d;
     if (ps.need_roadmap && !ps.direct) {
-        d.word = round_setup(ps, 0);
+        d.word = round_setup(ps);
         return d;
     }
     if (ps.need_roadmap) {  // single robot: no roadmap, start from the roots
@@ -1990,18 +2125,17 @@ __device__ PDecision after_step(PState &ps, bool accepted, unsigned long long no
     return PDecision{e.word, d.reset | e.reset};
 }
 
-__device__ PDecision decide(PState &ps, int kind, int r, unsigned long long now,
+__device__ PDecision decide(PState &ps, int kind, unsigned long long now,
                             unsigned long long deadline) {
     switch (kind) {
         case PK_BEGIN: return begin_outer(ps, now, deadline);
-        case PK_RM_SAMPLE: return {phase_word(PK_RM_VALC, r, chunks_of(ps.jobs[r].nc, kPerEdges)), 0};
-        case PK_RM_VALC: return {phase_word(PK_RM_APPEND, r, 1), 0};
-        case PK_RM_APPEND: return {phase_word(PK_RM_NB, r, chunks_of(ps.jobs[r].m, kPerWarps)), 0};
-        case PK_RM_NB: return {phase_word(PK_RM_EDGES, r, chunks_of(ps.jobs[r].emax, kPerThreads)), 0};
-        case PK_RM_EDGES: return {phase_word(PK_RM_VALE, r, chunks_of(ps.jobs[r].emax, kPerEdges)), 0};
-        case PK_RM_VALE: return {phase_word(PK_RM_LINK, r, 1), 0};
+        case PK_RM_SAMPLE: return {rm_word(ps, PK_RM_VALC), 0};
+        case PK_RM_VALC: return {rm_word(ps, PK_RM_APPEND), 0};
+        case PK_RM_APPEND: return {rm_word(ps, PK_RM_NB), 0};
+        case PK_RM_NB: return {rm_word(ps, PK_RM_EDGES), 0};
+        case PK_RM_EDGES: return {rm_word(ps, PK_RM_VALE), 0};
+        case PK_RM_VALE: return {rm_word(ps, PK_RM_LINK), 0};
         case PK_RM_LINK: {
-            if (r + 1 < ps.K) return {round_setup(ps, r + 1), 0};
             // the round is over for every robot (Alg. 2 ROADMAP)
             bool all = true;
             for (int k = 0; k < ps.K; ++k) all = all && *ps.jobs[k].conn != 0;
@@ -2024,23 +2158,23 @@ __device__ PDecision decide(PState &ps, int kind, int r, unsigned long long now,
             const PDecision e = end_outer(ps, now, deadline);
             return {e.word, d.reset | e.reset};
         }
-        case PK_ST_SAMPLE: return {phase_word(PK_ST_NN0, 0, kStepIters / kPQB), 0};
-        case PK_ST_NN0: return {phase_word(PK_ST_ORACLE, 0, 1), 0};
-        case PK_ST_ORACLE: return {phase_word(PK_ST_VAL1, 0, kStepIters / kPerEdges), 0};
-        case PK_ST_VAL1: return {phase_word(PK_ST_INSERT, 0, 1), 0};
-        case PK_ST_INSERT: return {phase_word(PK_ST_NN1, 0, kStepIters / kPQB), 0};
-        case PK_ST_NN1: return {phase_word(PK_ST_CONN, 0, 1), 0};
-        case PK_ST_CONN: return {phase_word(PK_ST_VAL2, 0, kStepIters / kPerEdges), 0};
-        case PK_ST_VAL2: return {phase_word(PK_ST_SOLUTION, 0, 1), 0};
+        case PK_ST_SAMPLE: return {phase_word(PK_ST_NN0, kStepIters / kPQB), 0};
+        case PK_ST_NN0: return {phase_word(PK_ST_ORACLE, 1), 0};
+        case PK_ST_ORACLE: return {phase_word(PK_ST_VAL1, kStepIters / kPerEdges), 0};
+        case PK_ST_VAL1: return {phase_word(PK_ST_INSERT, 1), 0};
+        case PK_ST_INSERT: return {phase_word(PK_ST_NN1, kStepIters / kPQB), 0};
+        case PK_ST_NN1: return {phase_word(PK_ST_CONN, 1), 0};
+        case PK_ST_CONN: return {phase_word(PK_ST_VAL2, kStepIters / kPerEdges), 0};
+        case PK_ST_VAL2: return {phase_word(PK_ST_SOLUTION, 1), 0};
         case PK_ST_SOLUTION:
-            if (ps.fine_M > 0) return {phase_word(PK_FINE_VAL, 0, chunks_of(ps.fine_cnt, kPerEdges)), 0};
+            if (ps.fine_M > 0) return {phase_word(PK_FINE_VAL, chunks_of(ps.fine_cnt, kPerEdges)), 0};
             return after_step(ps, false, now, deadline);
-        case PK_FINE_VAL: return {phase_word(PK_FINE_ACCEPT, 0, 1), 0};
+        case PK_FINE_VAL: return {phase_word(PK_FINE_ACCEPT, 1), 0};
         case PK_FINE_ACCEPT:
             if (ps.fine_bad) return after_step(ps, false, now, deadline);
-            if (!ps.accepted) return {phase_word(PK_FINE_VAL, 0, chunks_of(ps.fine_cnt, kPerEdges)), 0};
+            if (!ps.accepted) return {phase_word(PK_FINE_VAL, chunks_of(ps.fine_cnt, kPerEdges)), 0};
             return after_step(ps, true, now, deadline);
-        default: return {phase_word(PK_DONE, 0, 0), 0};
+        default: return {phase_word(PK_DONE, 0), 0};
     }
 }
 
@@ -2049,7 +2183,7 @@ __global__ void __launch_bounds__(kPerThreads) k_persistent(const PLaunch L) {
     __shared__ NnShared<kPerThreads> nn;
     __shared__ int wsum[kPerWarps];
     __shared__ double red[kPerThreads];
-    __shared__ int s_q, s_kind, s_robot, s_chunk, s_total, s_last, s_exit, s_next, s_reset;
+    __shared__ int s_q, s_kind, s_chunk, s_total, s_last, s_exit, s_next, s_reset;
     __shared__ unsigned long long s_t0, s_word;
     const int tid = threadIdx.x;
     if (tid == 0) {
@@ -2075,7 +2209,6 @@ __global__ void __launch_bounds__(kPerThreads) k_persistent(const PLaunch L) {
                 if (c >= tot) continue;
                 s_q = q;
                 s_kind = (int)(got >> 58);
-                s_robot = (int)((got >> 52) & 63);
                 s_total = tot;
                 s_chunk = c;
                 // the next claim starts at the next problem: the CTAs spread
@@ -2103,7 +2236,7 @@ __global__ void __launch_bounds__(kPerThreads) k_persistent(const PLaunch L) {
         __threadfence();  // acquire: the phase's inputs, written by other CTAs
         PState &ps = L.states[s_q];
         const unsigned long long tc0 = tid == 0 ? gtimer() : 0ull;
-        run_chunk(ps, s_kind, s_robot, s_chunk, per_sm4, nn, wsum, &s_next, red);
+        run_chunk(ps, s_kind, s_chunk, per_sm4, nn, wsum, &s_next, red);
         __threadfence();  // release: this chunk's results
         __syncthreads();
         if (tid == 0) {
@@ -2117,13 +2250,13 @@ __global__ void __launch_bounds__(kPerThreads) k_persistent(const PLaunch L) {
             const unsigned long long td0 = tid == 0 ? gtimer() : 0ull;
             if (tid == 0) {
                 const unsigned long long now = gtimer();
-                PDecision d = decide(ps, s_kind, s_robot, now, deadline);
+                PDecision d = decide(ps, s_kind, now, deadline);
                 // a phase without chunks (no new roadmap vertex to search
                 // around) is complete at once
                 for (int g = 0; g < 16; ++g) {
                     const int k2 = (int)(d.word >> 58);
                     if (k2 == PK_DONE || ((d.word >> 32) & 0xFFFFF) != 0) break;
-                    const PDecision d2 = decide(ps, k2, (int)((d.word >> 52) & 63), now, deadline);
+                    const PDecision d2 = decide(ps, k2, now, deadline);
                     d = PDecision{d2.word, d.reset | d2.reset};
                 }
                 s_word = d.word;
@@ -2277,7 +2410,8 @@ static mrpop_status plan_batch_persistent(mrpop_problem *const *ps, int n, doubl
     PL_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     cudaFuncAttributes fa{};
     PL_TRY(cudaFuncGetAttributes(&fa, k_persistent));
-    const size_t smem = std::max(need1, std::min(need8, (size_t)100 * 1024));
+    const size_t smem =
+        std::max({need1, std::min(need8, (size_t)100 * 1024), sizeof(LinkShared)});
     if (smem + fa.sharedSizeBytes > (size_t)optin)
         return set_error(MRPOP_EINVAL, "plan_batch: a problem's tables exceed the persistent "
                                        "kernel's shared memory (%zu bytes)", smem);
@@ -2306,7 +2440,7 @@ static mrpop_status plan_batch_persistent(mrpop_problem *const *ps, int n, doubl
         PState &s = hs[i];
         s = PState{};
         const bool act = run[i].active;
-        s.claim = act ? phase_word(PK_BEGIN, 0, 1) : phase_word(PK_DONE, 0, 0);
+        s.claim = act ? phase_word(PK_BEGIN, 1) : phase_word(PK_DONE, 0);
         s.finished = act ? 0 : 1;
         finished0 += act ? 0 : 1;
         s.mode = pl->mode;

@@ -305,8 +305,7 @@ mrpop_status mrpop_nearest(const float *tree, int64_t n_vertices, int64_t ld, in
                            int64_t *out_idx, void *cuda_stream);
 
 /* Filters of the large-batch NEAREST path (mrpop_nearest_ex).  Batches of
- * >= 2048 queries in dimensions 3, 6, 7, 14, 21 or 28 order the tree by g and
- * the queries by budget, then pass each (query, vertex) pair through an
+ * >= 2048 queries order the tree by g and the queries by budget, then pass each (query, vertex) pair through an
  * expansion filter |q|^2 + |x|^2 - 2 q.x <= bound, whose rounding error is
  * bounded so that it never drops the nearest admissible vertex; every vertex
  * that passes is decided with the exact FP32 distance, so the indices do not
@@ -316,8 +315,10 @@ mrpop_status mrpop_nearest(const float *tree, int64_t n_vertices, int64_t ld, in
  *   MRPOP_NEAREST_FILTER_TENSOR  the cross term on the tensor cores
  *                                (mma.sync: FP16 operands under an exact
  *                                power-of-two scaling for dim <= 14, TF32
- *                                above); a deliberate option beside the
- *                                FP32 path, faster on this GPU */
+ *                                above) in dimensions 3, 6, 7, 14, 21 and
+ *                                28 (others take the FP32 filter); a
+ *                                deliberate option beside the FP32 path,
+ *                                faster on this GPU */
 #define MRPOP_NEAREST_FILTER_FP32 0
 #define MRPOP_NEAREST_FILTER_TENSOR 1
 
@@ -330,9 +331,8 @@ mrpop_status mrpop_nearest_ex(const float *tree, int64_t n_vertices, int64_t ld,
 
 /* How many (query, vertex) pairs mrpop_nearest evaluates for these inputs
  * (a diagnostic for roofline accounting; no paper counterpart).  A vertex
- * with g_v >= c is never admissible, so for batches of >= 2048 queries in
- * dimensions 3, 6, 7, 14, 21 or 28 mrpop_nearest orders the tree by g and the
- * queries by budget and lets each block of 256 consecutive queries scan only
+ * with g_v >= c is never admissible, so for batches of >= 2048 queries
+ * mrpop_nearest orders the tree by g and the queries by budget and lets each block of 256 consecutive queries scan only
  * the vertices whose g bucket lies at or below its largest budget; other
  * batches scan all n_queries x n_vertices pairs.  Same arguments as
  * mrpop_nearest, with *pairs (host) receiving the count.  Synchronises the

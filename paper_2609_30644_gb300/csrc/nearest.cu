@@ -1291,6 +1291,7 @@ struct SortState {
     int gmin, gmax;                      // order-preserving keys of the finite g range
     int exact_only;                      // a coordinate lies outside the TF32 filter's range
     int nonfinite;                       // a coordinate is NaN or infinite
+    int neg_inf;                         // some g is -infinity (first bucket)
     unsigned maxabs;                     // largest finite coordinate magnitude (float bits)
     int arrive;                          // histogram blocks done (the last one scans)
     int tree_off[kSortBuckets + 1];      // bucket starts of the g-ordered tree
@@ -1306,9 +1307,10 @@ __device__ __forceinline__ int fkey(float v) {
 __device__ __forceinline__ float unkey(int o) { return __int_as_float(o ^ ((o >> 31) & 0x7fffffff)); }
 
 // Bucket of a value on the g scale; monotonic in v (a subtraction and a
-// product by a positive constant), non-finite values go to the last bucket.
+// product by a positive constant); -infinity goes to the first bucket, +infinity
+// and NaN to the last.
 __device__ __forceinline__ int sort_bucket(float v, float lo, float scale) {
-    if (!(fabsf(v) <= FLT_MAX)) return kSortBuckets - 1;
+    if (!(fabsf(v) <= FLT_MAX)) return v < 0.f ? 0 : kSortBuckets - 1;
     const float b = floorf((v - lo) * scale);
     if (!(b > 0.f)) return 0;
     return b >= (float)(kSortBuckets - 1) ? kSortBuckets - 1 : (int)b;
@@ -1360,6 +1362,7 @@ sort_setup(const float *__restrict__ g, int N, SortState *S, int *__restrict__ q
         S->gmax = hi;
         S->exact_only = 0;
         S->nonfinite = 0;
+        S->neg_inf = 0;
         S->maxabs = 0u;
         S->arrive = 0;
     }
@@ -1406,7 +1409,9 @@ sort_histogram(const float *__restrict__ g, int N, const float *__restrict__ c, 
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     float lo, scale;
     g_scale(*S, &lo, &scale);
-    grouped_add(S->tree_off + 1, i < N ? sort_bucket(g[i], lo, scale) : -1);
+    const float gi = i < N ? g[i] : 0.f;
+    if (gi == -INFINITY) S->neg_inf = 1;
+    grouped_add(S->tree_off + 1, i < N ? sort_bucket(gi, lo, scale) : -1);
     grouped_add(S->query_off + 1, i < Q ? sort_bucket(c[i], lo, scale) : -1);
     __threadfence();
     __syncthreads();
@@ -1448,8 +1453,10 @@ sort_histogram(const float *__restrict__ g, int N, const float *__restrict__ c, 
     }
 }
 
-// Scatter the tree (all D+1 rows) and the queries into bucket order.
-__global__ void sort_scatter(const float *__restrict__ tree, int N, int64_t ld, int dim,
+// Scatter the tree (all D+1 rows) and the queries into bucket order, in dp >=
+// dim coordinate rows of which the last dp - dim are zero (a zero coordinate
+// adds exactly nothing to a norm, a product chain or a distance).
+__global__ void sort_scatter(const float *__restrict__ tree, int N, int64_t ld, int dim, int dp,
                              const float *__restrict__ queries, const float *__restrict__ budgets,
                              int Q, SortState *S, float *__restrict__ tree_s, int ldt,
                              int *__restrict__ perm, float *__restrict__ q_s,
@@ -1471,17 +1478,17 @@ __global__ void sort_scatter(const float *__restrict__ tree, int N, int64_t ld, 
         if (a <= FLT_MAX) mx = max(mx, __float_as_uint(a));
     };
     if (i < N) {
-        // row dim + 1: the FP32 filter's folded squared norm fl(|x|^2) (1 - 4 gamma)
+        // row dp: g; row dp + 1: the FP32 filter's folded squared norm fl(|x|^2) (1 - 4 gamma)
         float n2 = 0.f;
-        for (int d = 0; d <= dim; ++d) {
+        for (int d = 0; d < dim; ++d) {
             const float v = tree[(size_t)d * ld + i];
-            if (d < dim) {
-                check(v);
-                n2 = fmaf(v, v, n2);
-            }
+            check(v);
+            n2 = fmaf(v, v, n2);
             tree_s[(size_t)d * ldt + pt] = v;
         }
-        tree_s[(size_t)(dim + 1) * ldt + pt] = n2 * (1.f - 4.f * (kF32G * (dim + 2.f)));
+        for (int d = dim; d < dp; ++d) tree_s[(size_t)d * ldt + pt] = 0.f;
+        tree_s[(size_t)dp * ldt + pt] = tree[(size_t)dim * ld + i];
+        tree_s[(size_t)(dp + 1) * ldt + pt] = n2 * (1.f - 4.f * (kF32G * (dp + 2.f)));
         perm[pt] = i;
     }
     const float c = i < Q ? budgets[i] : 0.f;
@@ -1493,6 +1500,7 @@ __global__ void sort_scatter(const float *__restrict__ tree, int N, int64_t ld, 
             check(v);
             q_s[(size_t)d * Q + pq] = v;
         }
+        for (int d = dim; d < dp; ++d) q_s[(size_t)d * Q + pq] = 0.f;
         c_s[pq] = c;
         qperm[pq] = i;
     }
@@ -1523,10 +1531,9 @@ __global__ void __launch_bounds__(256) sort_cut(const float *__restrict__ c_s, i
         float lo, scale;
         g_scale(*S, &lo, &scale);
         int n;
-        if (S->gmin > S->gmax)
-            n = 0;                                 // no finite g at all
-        else if (!(m > unkey(S->gmin)))
-            n = 0;                                 // no vertex has g < m
+        if (S->gmin > S->gmax || !(m > unkey(S->gmin)))
+            // no finite g at all, or none below m
+            n = S->neg_inf ? S->tree_off[1] : 0;
         else if (m > unkey(S->gmax))
             n = N;
         else
@@ -1589,10 +1596,9 @@ nearest_seed(const float *__restrict__ tree_s, int N, int ldt, const float *__re
         float lo, scale;
         g_scale(*S, &lo, &scale);
         int nc;
-        if (S->gmin > S->gmax)
-            nc = 0;                                 // no finite g at all
-        else if (!(m > unkey(S->gmin)))
-            nc = 0;                                 // no vertex has g < m
+        if (S->gmin > S->gmax || !(m > unkey(S->gmin)))
+            // no finite g at all, or none below m
+            nc = S->neg_inf ? S->tree_off[1] : 0;
         else if (m > unkey(S->gmax))
             nc = N;
         else
@@ -1634,27 +1640,33 @@ mrpop_status f32_filter_setup(int dev, int *bps) {
     return MRPOP_OK;
 }
 
+// Dimensions of the tensor-core filters' instances; the FP32 filter serves the
+// padded dimensions between and above them whatever the filter asked for.
+constexpr bool tensor_dim(int d) {
+    return d == 3 || d == 6 || d == 7 || d == 14 || d == 21 || d == 28;
+}
+
+// DIM: the instance's coordinate rows, dim <= DIM of them the caller's.
 // out_idx null: only count the scanned pairs into *pairs (synchronises).
 // filter: MRPOP_NEAREST_FILTER_FP32 (FMA-pipe expansion filter) or
 // MRPOP_NEAREST_FILTER_TENSOR (FP16 / TF32 mma.sync expansion filter); both
 // decide every survivor exactly, so the indices do not depend on it.
 template <int DIM>
-mrpop_status nearest_sorted(const float *tree, int N, int64_t ld, const float *queries,
-                                const float *budgets, int Q, int64_t *out_idx, cudaStream_t st,
-                                int64_t *pairs = nullptr, int filter = MRPOP_NEAREST_FILTER_FP32,
-                                int waves = 4) {
+mrpop_status nearest_sorted(const float *tree, int N, int64_t ld, int dim, const float *queries,
+                            const float *budgets, int Q, int64_t *out_idx, cudaStream_t st,
+                            int64_t *pairs, int filter, int waves) {
     int dev = 0, sms = 1, bps = 1;
     MRPOP_CUDA_TRY(cudaGetDevice(&dev));
     MRPOP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     constexpr bool f16 = DIM + 2 <= 16;  // FP16 tensor filter (K = 16), else TF32
-    const bool tensor = filter == MRPOP_NEAREST_FILTER_TENSOR;
+    const bool tensor = tensor_dim(DIM) && dim == DIM && filter == MRPOP_NEAREST_FILTER_TENSOR;
     if (!tensor) {
         const mrpop_status fs = f32_filter_setup<DIM>(dev, &bps);
         if (fs != MRPOP_OK) return fs;
-    } else if constexpr (f16) {
+    } else if constexpr (tensor_dim(DIM) && f16) {
         MRPOP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, nearest_tc16_kernel<DIM>,
                                                                      kTcThreads, 0));
-    } else {
+    } else if constexpr (tensor_dim(DIM)) {
         MRPOP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, nearest_tc_kernel<DIM>,
                                                                      kTcThreads, 0));
     }
@@ -1686,10 +1698,14 @@ mrpop_status nearest_sorted(const float *tree, int N, int64_t ld, const float *q
     const size_t b_seed = align(sizeof(float) * (size_t)Q);
     const size_t b_qdone = align(sizeof(int) * (size_t)qblocks);
     char *arena = nullptr;
-    MRPOP_CUDA_TRY(scratch_alloc((void **)&arena,
-                                   b_state + b_tree + b_perm + b_q + b_c + b_qp + b_cut + b_part +
-                                       b_seed + b_qdone,
-                                   st));
+    const cudaError_t ae = scratch_alloc((void **)&arena,
+                                         b_state + b_tree + b_perm + b_q + b_c + b_qp + b_cut +
+                                             b_part + b_seed + b_qdone,
+                                         st);
+    if (ae != cudaSuccess) {
+        cudaGetLastError();  // not left for a later launch check
+        return cuda_error(ae, "nearest: scratch");
+    }
     char *at = arena;
     auto take = [&](size_t b) { char *r = at; at += b; return r; };
     SortState *S = (SortState *)take(b_state);
@@ -1703,7 +1719,7 @@ mrpop_status nearest_sorted(const float *tree, int N, int64_t ld, const float *q
     float *seed = (float *)take(b_seed);
     int *qdone = (int *)take(b_qdone);
     const int n_max = std::max(N, Q);
-    const float *g = tree + (size_t)DIM * ld;
+    const float *g = tree + (size_t)dim * ld;
     // five launches: setup (+ range), histogram (+ scan), scatter, seed (+
     // cut), filter (+ reduce in each query block's last slice)
     const bool setup_range = N <= kSetupRangeMax;
@@ -1711,8 +1727,8 @@ mrpop_status nearest_sorted(const float *tree, int N, int64_t ld, const float *q
     if (!setup_range) sort_range<<<(N + 255) / 256, 256, 0, st>>>(g, N, S);
     sort_histogram<<<(n_max + kHistThreads - 1) / kHistThreads, kHistThreads, 0, st>>>(
         g, N, budgets, Q, S);
-    sort_scatter<<<(n_max + 255) / 256, 256, 0, st>>>(tree, N, ld, DIM, queries, budgets, Q, S,
-                                                       tree_s, ldt, perm, q_s, c_s, qperm);
+    sort_scatter<<<(n_max + 255) / 256, 256, 0, st>>>(tree, N, ld, dim, DIM, queries, budgets, Q,
+                                                       S, tree_s, ldt, perm, q_s, c_s, qperm);
     if (!out_idx) {
         sort_cut<<<qblocks, 256, 0, st>>>(c_s, Q, bq, S, N, cut);
         unsigned long long *d_pairs = (unsigned long long *)seed;  // 8 bytes of the arena
@@ -1733,11 +1749,11 @@ mrpop_status nearest_sorted(const float *tree, int N, int64_t ld, const float *q
     if (!tensor)
         nearest_f32_kernel<DIM><<<grid, kTcThreads, f32_smem_bytes<DIM>(), st>>>(
             tree_s, N, ldt, q_s, c_s, Q, chunk, partial, perm, cut, seed, &S->exact_only, fin);
-    else if constexpr (f16)
+    else if constexpr (tensor_dim(DIM) && f16)
         nearest_tc16_kernel<DIM><<<grid, kTcThreads, 0, st>>>(tree_s, N, ldt, q_s, c_s, Q, chunk,
                                                               partial, perm, cut, seed,
                                                               &S->maxabs, &S->nonfinite, fin);
-    else
+    else if constexpr (tensor_dim(DIM))
         nearest_tc_kernel<DIM><<<grid, kTcThreads, 0, st>>>(tree_s, N, ldt, q_s, c_s, Q, chunk, partial,
                                                             perm, cut, seed, &S->exact_only, fin);
     const cudaError_t e = cudaGetLastError();
@@ -1953,25 +1969,59 @@ mrpop_status autotune_neighbors(const float *tree, int64_t N, int64_t ld, int di
                            st, target_out, ms_out);
 }
 
+// The budget-ordered path at the smallest instance of at least dim rows.  Its
+// own instance for the dimensions of this library's arms and their first
+// multiples, steps of 4 to 12 rows elsewhere: the chain of a pair is as long
+// as the rows, so padding costs (DIM - dim) / dim of it, where the exact scan
+// these dimensions took before costs two operations per coordinate of all
+// N Q pairs, read from L2 once per 8 queries (35-D, 8,192 queries over 50,000
+// vertices: 2,457 us against 501).
+static mrpop_status nearest_sorted_dim(const float *tree, int n, int64_t ld, int dim,
+                                       const float *queries, const float *budgets, int q,
+                                       int64_t *out_idx, cudaStream_t st, int64_t *pairs,
+                                       int filter, int w) {
+#define MRPOP_NN_DIM(D)                                                                       \
+    if (dim <= D)                                                                             \
+        return nearest_sorted<D>(tree, n, ld, dim, queries, budgets, q, out_idx, st, pairs, filter, w)
+    MRPOP_NN_DIM(3);
+    MRPOP_NN_DIM(6);
+    MRPOP_NN_DIM(7);
+    MRPOP_NN_DIM(12);
+    MRPOP_NN_DIM(14);
+    MRPOP_NN_DIM(16);
+    MRPOP_NN_DIM(21);
+    MRPOP_NN_DIM(24);
+    MRPOP_NN_DIM(28);
+    MRPOP_NN_DIM(32);
+    MRPOP_NN_DIM(36);
+    MRPOP_NN_DIM(44);
+    MRPOP_NN_DIM(52);
+    MRPOP_NN_DIM(56);
+    MRPOP_NN_DIM(64);
+#undef MRPOP_NN_DIM
+    return set_error(MRPOP_EINVAL, "nearest: dimension %d", dim);
+}
+
+// Whether a call takes the budget-ordered path.
+static bool takes_sorted(int dim, int64_t N, int64_t Q) {
+    return Q >= 2048 && N > 0 && (N <= (1 << 30) || tensor_dim(dim));
+}
+
 mrpop_status launch_nearest(const float *tree, int64_t N, int64_t ld, int dim,
                             const float *queries, const float *budgets, int64_t Q,
                             int64_t *out_idx, cudaStream_t st, int filter, int waves) {
     const int n = (int)N, q = (int)Q;
     // Large batches: budget-ordered tree and queries, expansion filter with
     // exact decisions over shared-memory tree tiles.
-    if (Q >= 2048 && N > 0) {
+    if (takes_sorted(dim, N, Q)) {
         const int w = waves > 0 ? waves : nearest_tuned(dim, N, Q, filter);
-        switch (dim) {
-            case 3: return nearest_sorted<3>(tree, n, ld, queries, budgets, q, out_idx, st, nullptr, filter, w);
-            case 6: return nearest_sorted<6>(tree, n, ld, queries, budgets, q, out_idx, st, nullptr, filter, w);
-            case 7: return nearest_sorted<7>(tree, n, ld, queries, budgets, q, out_idx, st, nullptr, filter, w);
-            case 14: return nearest_sorted<14>(tree, n, ld, queries, budgets, q, out_idx, st, nullptr, filter, w);
-            case 21: return nearest_sorted<21>(tree, n, ld, queries, budgets, q, out_idx, st, nullptr, filter, w);
-            case 28: return nearest_sorted<28>(tree, n, ld, queries, budgets, q, out_idx, st, nullptr, filter, w);
-            default: break;
-        }
+        const mrpop_status s = nearest_sorted_dim(tree, n, ld, dim, queries, budgets, q, out_idx,
+                                                  st, nullptr, filter, w);
+        // the ordered copies of a tree that nearly fills the device did not
+        // fit: the scan below needs none
+        if (s != MRPOP_ENOMEM) return s;
     }
-    // Small batches (and other dimensions): vertices across lanes, queries
+    // Small batches: vertices across lanes, queries
     // broadcast from shared memory, warp-shuffle argmin.
     const int dp = (dim + 3) & ~3;
     switch (dp) {
@@ -1993,17 +2043,9 @@ mrpop_status nearest_pairs(const float *tree, int64_t N, int64_t ld, int dim, co
                            const float *budgets, int64_t Q, int64_t *pairs, cudaStream_t st) {
     const int n = (int)N, q = (int)Q;
     *pairs = N * Q;  // the small-batch kernels scan every vertex
-    if (Q >= 2048 && N > 0) {
-        switch (dim) {
-            case 3: return nearest_sorted<3>(tree, n, ld, queries, budgets, q, nullptr, st, pairs);
-            case 6: return nearest_sorted<6>(tree, n, ld, queries, budgets, q, nullptr, st, pairs);
-            case 7: return nearest_sorted<7>(tree, n, ld, queries, budgets, q, nullptr, st, pairs);
-            case 14: return nearest_sorted<14>(tree, n, ld, queries, budgets, q, nullptr, st, pairs);
-            case 21: return nearest_sorted<21>(tree, n, ld, queries, budgets, q, nullptr, st, pairs);
-            case 28: return nearest_sorted<28>(tree, n, ld, queries, budgets, q, nullptr, st, pairs);
-            default: break;
-        }
-    }
+    if (takes_sorted(dim, N, Q))
+        return nearest_sorted_dim(tree, n, ld, dim, queries, budgets, q, nullptr, st, pairs,
+                                  MRPOP_NEAREST_FILTER_FP32, 4);
     return MRPOP_OK;
 }
 

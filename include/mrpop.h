@@ -304,8 +304,11 @@ mrpop_status mrpop_nearest(const float *tree, int64_t n_vertices, int64_t ld, in
                            const float *queries, const float *budgets, int64_t n_queries,
                            int64_t *out_idx, void *cuda_stream);
 
-/* Filters of the large-batch NEAREST path (mrpop_nearest_ex).  Batches of
- * >= 2048 queries order the tree by g and the queries by budget, then pass each (query, vertex) pair through an
+/* Filters of the large-batch NEAREST path (mrpop_nearest_ex).  Large batches
+ * (by the product of queries, vertices and dimensions; always from 4,096
+ * queries over 2,560 vertices, and from 2,048 queries with the tensor-core
+ * filter) order the tree by g and the queries by budget, then pass each
+ * (query, vertex) pair through an
  * expansion filter |q|^2 + |x|^2 - 2 q.x <= bound, whose rounding error is
  * bounded so that it never drops the nearest admissible vertex; every vertex
  * that passes is decided with the exact FP32 distance, so the indices do not
@@ -331,8 +334,9 @@ mrpop_status mrpop_nearest_ex(const float *tree, int64_t n_vertices, int64_t ld,
 
 /* How many (query, vertex) pairs mrpop_nearest evaluates for these inputs
  * (a diagnostic for roofline accounting; no paper counterpart).  A vertex
- * with g_v >= c is never admissible, so for batches of >= 2048 queries
- * mrpop_nearest orders the tree by g and the queries by budget and lets each block of 256 consecutive queries scan only
+ * with g_v >= c is never admissible, so for large batches (see above, with the
+ * default filter) mrpop_nearest orders the tree by g and the queries by budget
+ * and lets each block of 256 consecutive queries scan only
  * the vertices whose g bucket lies at or below its largest budget; other
  * batches scan all n_queries x n_vertices pairs.  Same arguments as
  * mrpop_nearest, with *pairs (host) receiving the count.  Synchronises the

@@ -37,7 +37,8 @@ def _inputs(D, n, Q, seed):
     k = min(n // 4, 40)
     tree[:, n - k:n] = tree[:, :k]
     tree[D, n - k:n - k // 2] += np.float32(0.5)
-    qs[:, :k] = tree[:D, :k]
+    kq = min(k, Q)
+    qs[:, :kq] = tree[:D, :kq]
     return tree, qs, cs
 
 
@@ -46,7 +47,7 @@ def _inputs(D, n, Q, seed):
 @pytest.mark.parametrize("D", [1, 2, 4, 5, 8, 12, 13, 15, 16, 17, 21, 22, 24, 25, 29, 32, 33, 35,
                                36, 37, 42, 44, 45, 49, 52, 53, 56, 57, 63, 64])
 def test_large_batches_in_every_dimension(mp, D):
-    n, Q = 3001, 2100
+    n, Q = 3001, 4100
     tree, qs, cs = _inputs(D, n, Q, D)
     t, q, c = _dev(tree), _dev(qs), _dev(cs)
     want = _scan(mp, t, q, c, n)
@@ -57,9 +58,10 @@ def test_large_batches_in_every_dimension(mp, D):
 
 @pytest.mark.parametrize("D", [14, 35])
 @pytest.mark.parametrize("what", ["inf_g", "neg_inf_g", "all_neg_inf_g", "inf_budget",
-                                  "nan", "huge", "lowest", "equal_g"])
+                                  "nan", "huge", "lowest", "equal_g", "offset", "tiny",
+                                  "colossal", "scaled_down", "scaled_up"])
 def test_large_batches_of_extreme_values(mp, D, what):
-    n, Q = 2500, 2048
+    n, Q = 2600, 4096
     tree, qs, cs = _inputs(D, n, Q, 7)
     if what == "inf_g":
         tree[D, ::3] = np.inf
@@ -80,6 +82,40 @@ def test_large_batches_of_extreme_values(mp, D, what):
         cs[::2] = np.finfo(np.float32).min
     elif what == "equal_g":
         tree[D] = np.float32(1.5)
+    elif what == "offset":              # large norms, small distances
+        tree[:D] += np.float32(1000.0)
+        qs += np.float32(1000.0)
+    elif what == "tiny":                # below the filter's range: every pair decided exactly
+        qs[3, 5] = np.float32(1e-25)
+    elif what == "colossal":            # -2 q overflows
+        qs[2, 9] = tree[2, 9] = np.float32(3e38)
+        cs[9] = tree[D, 9] + np.float32(1.0)
+    elif what in ("scaled_down", "scaled_up"):
+        for a in (tree, qs, cs):
+            a *= np.float32(1e-12 if what == "scaled_down" else 1e15)
     t, q, c = _dev(tree), _dev(qs), _dev(cs)
     torch.testing.assert_close(mp.nearest(t, q, c, n_vertices=n), _scan(mp, t, q, c, n),
                                rtol=0, atol=0)
+
+
+# the scan's routes: one slice, a cluster of slices, slices with a second
+# kernel; rows of 6, 7 and 8 with and without padding; ragged query tiles,
+# steps and rows that are not 16-byte aligned
+@pytest.mark.parametrize("D,n,Q", [(6, 1, 1), (7, 255, 64), (8, 257, 65), (9, 1023, 63), (14, 2048, 2),
+                                   (13, 2049, 130), (28, 5003, 257), (35, 20001, 40), (64, 3001, 70),
+                                   (3, 999, 2500), (1, 4000, 300)])
+def test_scan_against_oracle(mp, orc, D, n, Q):
+    tree, qs, cs = _inputs(D, n, Q, D + n) if n > 4 else (
+        np.zeros((D + 1, 6), np.float32), np.ones((D, Q), np.float32), np.full(Q, 9.0, np.float32))
+    t, q, c = _dev(tree), _dev(qs), _dev(cs)
+    got = mp.nearest(t, q, c, n_vertices=n).cpu().numpy()
+    noalloc = torch.full((Q,), -7, dtype=torch.int64, device="cuda")
+    assert mp.lib.mrpop_nearest_noalloc(t.data_ptr(), n, tree.shape[1], D, q.data_ptr(),
+                                        c.data_ptr(), Q, noalloc.data_ptr(),
+                                        torch.cuda.current_stream().cuda_stream) == 0
+    np.testing.assert_array_equal(noalloc.cpu().numpy(), got)
+    for i in range(0, Q, max(1, Q // 60)):
+        ref, bd, sd, gap = orc.nearest(tree, qs[:, i], cs[i], n_vertices=n)
+        # a different vertex only where FP32 cannot tell the two apart
+        assert got[i] == ref or (np.isfinite(sd) and sd - bd <= 1e-5 * max(bd, 1e-30)) or \
+            gap <= 1e-5 * max(1.0, abs(float(cs[i]))), (i, got[i], ref)

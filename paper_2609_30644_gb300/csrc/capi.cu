@@ -176,10 +176,74 @@ static void coarse_sphere(const float *xyzr, int n, float out[4]) {
     out[3] = (float)(r + 1e-4);
 }
 
+// Places the distance field of p's obstacles: sets p->dev.t's df_* fields
+// except df, and its own parameters; no voxels when there are no obstacles
+// within reach (nothing can touch them), or, with df_out 0 (every look-up
+// says near), when the coordinates are too large for the index arithmetic.
+// hi: a corner above every reachable coarse centre, as ws_lo is one below.
+static bool place_field(Tables &t, const std::vector<float> &blob, const double *hi, double max_th,
+                        float *edge_out, float *shrink_out) {
+    double lo[3], up[3], big = 0.0;
+    for (int a = 0; a < 3; ++a) lo[a] = HUGE_VAL, up[a] = -HUGE_VAL;
+    auto f4 = [&](int i) { return blob.data() + 4 * (size_t)i; };
+    auto add = [&](const float *c, double r) {
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = std::min(lo[a], (double)c[a] - r);
+            up[a] = std::max(up[a], (double)c[a] + r);
+        }
+    };
+    for (int o = 0; o < t.NS; ++o) add(f4(t.off_os + o), f4(t.off_os + o)[3]);
+    for (int o = 0; o < t.NC; ++o) add(f4(t.off_oc + kCuboidF4 * o), f4(t.off_oc + kCuboidF4 * o)[3]);
+    t.df_out = 255;
+    if (!(max_th > 0.0) || t.NS + t.NC == 0) return false;
+    // a voxel edge of an eighth of the largest threshold, longer when the box
+    // would need more than kFieldMaxVoxels
+    double edge = max_th / 8.0;
+    for (int pass = 0; pass < 64; ++pass) {
+        double voxels = 1.0;
+        int first[3];
+        bool fits = true;
+        for (int a = 0; a < 3; ++a) {
+            const double pad = max_th + 2.0 * edge;
+            const double l = std::max(lo[a] - pad, (double)t.ws_lo[a]);
+            const double u = std::min(up[a] + pad, hi[a]);
+            if (!(l <= u)) return false;  // nothing within reach along this axis
+            big = std::max({big, std::fabs(l), std::fabs(u)});
+            const double i0 = std::floor(l / edge), n = std::ceil(u / edge) - i0 + 1.0;
+            fits = fits && std::fabs(i0) + n < 2e6;
+            first[a] = fits ? (int)i0 : 0;
+            t.df_n[a] = fits ? (int)n : 0;
+            voxels *= n;
+        }
+        if (!fits || voxels > kFieldMaxVoxels) {
+            edge *= std::max(1.01, std::cbrt(std::min(voxels, 1e18) / kFieldMaxVoxels));
+            continue;
+        }
+        t.df_inv = (float)(1.0 / edge);
+        for (int a = 0; a < 3; ++a) t.df_c[a] = kFieldMagic - (float)first[a];
+        // half a voxel's diagonal; FP32 rounding of coordinates up to big, of
+        // the look-up's index (a relative 2^-23 of the coordinate) and of the
+        // bound itself
+        *edge_out = (float)edge;
+        *shrink_out = (float)(edge * 0.5 * 1.7320509 + 4e-4 + 1e-3 * edge + 8e-7 * big);
+        return true;
+    }
+    for (int a = 0; a < 3; ++a) t.df_n[a] = 0;
+    t.df_out = 0;
+    return false;
+}
+
 extern "C" mrpop_status mrpop_create_problem(const mrpop_robot *robots, int32_t K,
                                              const mrpop_obstacles *obs, const float *start,
                                              const float *goal, const mrpop_config *cfg,
                                              mrpop_problem **out) {
+    return create_problem(robots, K, obs, start, goal, cfg, nullptr, out);
+}
+
+mrpop_status mrpop::create_problem(const mrpop_robot *robots, int32_t K,
+                                   const mrpop_obstacles *obs, const float *start,
+                                   const float *goal, const mrpop_config *cfg,
+                                   const mrpop_problem *share, mrpop_problem **out) {
     if (!out) return set_error(MRPOP_EINVAL, "mrpop_create_problem: out is NULL");
     *out = nullptr;
     if (!robots || !obs || !cfg)
@@ -311,9 +375,10 @@ extern "C" mrpop_status mrpop_create_problem(const mrpop_robot *robots, int32_t 
         std::memcpy(f4(t.off_sph + s_glob), r.sphere_xyzr, 4 * sizeof(float) * r.n_spheres);
         s_glob += r.n_spheres;
     }
-    // workspace corner below every reachable coarse centre: |origin_j - base|
-    // <= sum_i |(a_i, 0, d_i)| along the chain, |coarse centre - origin_j| <=
-    // the largest coarse-centre offset of the robot
+    // workspace corners below and above every reachable coarse centre:
+    // |origin_j - base| <= sum_i |(a_i, 0, d_i)| along the chain, |coarse
+    // centre - origin_j| <= the largest coarse-centre offset of the robot
+    double ws_hi[3] = {-HUGE_VAL, -HUGE_VAL, -HUGE_VAL}, max_th = 0.0;
     {
         double lo[3] = {HUGE_VAL, HUGE_VAL, HUGE_VAL};
         for (int k = 0; k < K; ++k) {
@@ -325,7 +390,10 @@ extern "C" mrpop_status mrpop_create_problem(const mrpop_robot *robots, int32_t 
                 const float *A = f4(t.off_link + kLinkF4 * (t.link0[k] + j)) + 8;
                 off = std::max(off, std::sqrt((double)A[0] * A[0] + (double)A[1] * A[1] +
                                               (double)A[2] * A[2]));
+                if (A[3] > 0.f) max_th = std::max(max_th, (double)A[3] + cfg->margin);
             }
+            for (int a = 0; a < 3; ++a)
+                ws_hi[a] = std::max(ws_hi[a], (double)r.base[4 * a + 3] + reach + off);
             for (int a = 0; a < 3; ++a)
                 lo[a] = std::min(lo[a], (double)r.base[4 * a + 3] - reach - off);
         }
@@ -350,9 +418,45 @@ extern "C" mrpop_status mrpop_create_problem(const mrpop_robot *robots, int32_t 
         }
     }
 
+    // the distance field and the links' thresholds in its unit
+    float edge = 0.f, shrink = 0.f;
+    bool build = false;
+    double unit = max_th / 240.0;
+    if (share) {
+        const Tables &o = share->dev.t;
+        t.df = o.df;
+        t.df_out = o.df_out;
+        t.df_inv = o.df_inv;
+        for (int a = 0; a < 3; ++a) t.df_n[a] = o.df_n[a], t.df_c[a] = o.df_c[a];
+        unit = share->field_unit;
+    } else {
+        build = place_field(t, blob, ws_hi, max_th, &edge, &shrink);
+    }
+    for (int l = 0; l < L; ++l) {
+        const float *A = f4(t.off_link + kLinkF4 * l);
+        int cnt;
+        std::memcpy(&cnt, A + 6, sizeof(cnt));
+        // a link without spheres touches nothing: threshold 0
+        const double th = cnt > 0 && unit > 0.0
+                              ? std::ceil(((double)A[11] + cfg->margin) / unit * (1.0 + 1e-6)) : 0.0;
+        f4(t.off_link + kLinkF4 * l + 3)[0] = f_of_i((int)std::min(th, 255.0));
+        f4(t.off_link + kLinkF4 * l + 3)[2] = l + 1 < L ? f4(t.off_link + kLinkF4 * (l + 1))[4] : 0.f;
+    }
+    for (int k = 0; k < K; ++k) {  // each robot's largest coarse radius (-1: no spheres)
+        float rmax = -1.f;
+        for (int l = t.link0[k]; l < t.link0[k + 1]; ++l) {
+            const float *A = f4(t.off_link + kLinkF4 * l);
+            int cnt;
+            std::memcpy(&cnt, A + 6, sizeof(cnt));
+            if (cnt > 0) rmax = std::max(rmax, A[11]);
+        }
+        for (int l = t.link0[k]; l < t.link0[k + 1]; ++l) f4(t.off_link + kLinkF4 * l + 3)[1] = rmax;
+    }
+
     mrpop_problem *p = new (std::nothrow) mrpop_problem();
     if (!p) return set_error(MRPOP_ENOMEM, "host allocation failed");
     p->dev.t = t;
+    p->field_unit = unit;
     p->cfg = *cfg;
     p->D = L;
     p->h_blob.swap(blob);
@@ -397,6 +501,15 @@ extern "C" mrpop_status mrpop_create_problem(const mrpop_robot *robots, int32_t 
     if ((e = cudaMemcpy(p->dev.blob, p->h_blob.data(), p->h_blob.size() * sizeof(float),
                         cudaMemcpyHostToDevice)) != cudaSuccess)
         return fail(cuda_error(e, "cudaMemcpy(tables)"));
+    if (build) {
+        const size_t voxels = (size_t)t.df_n[0] * t.df_n[1] * t.df_n[2];
+        if ((e = cudaMalloc(&p->dev.field, voxels)) != cudaSuccess)
+            return fail(cuda_error(e, "cudaMalloc(distance field)"));
+        p->dev.t.df = p->dev.field;
+        const mrpop_status s =
+            launch_field(p->dev.t, p->dev.blob, edge, shrink, (float)unit, p->dev.field, nullptr);
+        if (s != MRPOP_OK) return fail(s);
+    }
     if ((e = cudaMalloc(&p->dev.q_lo, sizeof(float) * L)) != cudaSuccess ||
         (e = cudaMalloc(&p->dev.q_hi, sizeof(float) * L)) != cudaSuccess)
         return fail(cuda_error(e, "cudaMalloc(limits)"));
@@ -408,6 +521,9 @@ extern "C" mrpop_status mrpop_create_problem(const mrpop_robot *robots, int32_t 
         return fail(cuda_error(e, "cudaMalloc(counter)"));
     if ((e = cudaMemset(p->dev.edge_counter, 0, sizeof(int) * 4)) != cudaSuccess)
         return fail(cuda_error(e, "cudaMemset(counter)"));
+    // the field and the counter are used on any stream from here on
+    if ((e = cudaStreamSynchronize(nullptr)) != cudaSuccess)
+        return fail(cuda_error(e, "problem tables"));
     // a launch tuned earlier for a problem of this shape (mrpop_autotune)
     std::vector<int> tuned;
     if (tune_lookup(validate_tune_key(p), &tuned) && tuned.size() >= 4) {
@@ -426,6 +542,7 @@ extern "C" mrpop_status mrpop_destroy_problem(mrpop_problem *p) {
     destroy_planner(p->planner);
     p->planner = nullptr;
     cudaFree(p->dev.blob);
+    cudaFree(p->dev.field);
     cudaFree(p->dev.q_lo);
     cudaFree(p->dev.q_hi);
     cudaFree(p->dev.edge_counter);

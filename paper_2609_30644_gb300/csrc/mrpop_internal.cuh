@@ -16,9 +16,13 @@ namespace mrpop {
 // in one contiguous float4 blob that each block stages into shared memory:
 //
 //   base     K x 3 float4   rows of the 3x4 base pose [R | t]
-//   link     L x 3 float4   (a, d, cos alpha, sin alpha)
-//                           (theta_offset, first sphere, sphere count, robot)
+//   link     L x 4 float4   (a, d, cos alpha, sin alpha)
+//                           (theta_offset, first sphere, sphere count,
+//                            same-robot partner bits)
 //                           (coarse centre x, y, z in F_j', coarse radius)
+//                           (distance-field threshold, the robot's largest
+//                            coarse radius or -1, theta_offset of the next
+//                            link or 0, 0)
 //   sphere   S x 1 float4   (x, y, z in F_j', r), grouped by link
 //   osphere  NS x 1 float4  (cx, cy, cz, r)
 //   cuboid   NC x 5 float4  (cx, cy, cz, bounding radius |h|), (hx, hy, hz, 0),
@@ -38,9 +42,28 @@ struct Tables {
     // 1 m): coordinates taken relative to it are >= 0, so their float bits
     // order like unsigned integers.
     float ws_lo[3] = {0.f, 0.f, 0.f};
+    // Distance field of the obstacles (DistanceField below).
+    const uint8_t *df = nullptr;  // [df_n[2]][df_n[1]][df_n[0]], device
+    int df_n[3] = {0, 0, 0};      // voxels per axis (0: none)
+    int df_out = 255;             // value outside the field
+    float df_inv = 0.f;           // 1 / voxel edge
+    float df_c[3] = {0.f, 0.f, 0.f};  // kFieldMagic minus the first voxel's index
 };
 
-constexpr int kLinkF4 = 3;
+// Distance field of a problem's obstacles: a box of cubic voxels, one byte
+// each, around everything that a link's coarse sphere could touch.  A voxel
+// holds a lower bound of the distance from any point in it to the nearest
+// obstacle, in units of a 240th of the largest coarse radius plus margin
+// (rounded down), so that one byte load tells that a link's coarse sphere is
+// clear of every obstacle: value >= the link's threshold (rounded up).  Voxel
+// i along an axis is centred on i voxel edges, so the index is the coordinate
+// in voxel edges rounded to nearest: fmaf(x, 1 / edge, kFieldMagic - first),
+// whose low mantissa bits are the index.
+constexpr float kFieldMagic = 12582912.f;      // 1.5 * 2^23
+constexpr int kFieldMagicBits = 0x4b400000;    // its bit pattern
+constexpr int kFieldMaxVoxels = 1 << 19;
+
+constexpr int kLinkF4 = 4;
 constexpr int kCuboidF4 = 5;
 // Kept per stored link and checkpoint for later links' robot-robot tests: the
 // link's coarse sphere centre (3 floats); the rare fine tests rebuild the
@@ -81,8 +104,18 @@ inline int validate_warp_floats(const Tables &t, int fine) {
     return 2 * dpad + 4 * nstore + nstore * kXcFloats * 32 + (fine ? kFrFloats * 32 + 64 : 0);
 }
 
+// Per-warp shared scratch of the verdict body (floats): (q_a, q_b - q_a) of
+// every joint and a spare one, the robots' tile boxes and the coarse centres of
+// every link.
+inline int verdict_dpad(const Tables &t) { return (t.L + 4) & ~3; }
+inline int verdict_warp_floats(const Tables &t) {
+    const int dpad = verdict_dpad(t);
+    return 2 * dpad + 8 * t.K + t.L * kXcFloats * 32;
+}
+
 struct DeviceProblem {
     Tables t;
+    uint8_t *field = nullptr;     // the distance field where this problem owns it
     float4 *blob = nullptr;       // device copy of the table blob
     float *q_lo = nullptr;        // device [D]
     float *q_hi = nullptr;        // device [D]
@@ -114,6 +147,7 @@ struct mrpop_problem {
     std::vector<float> start, goal, q_lo, q_hi;
     int num_sms = 0;
     size_t smem_optin = 0;
+    double field_unit = 0.0;  // metres per unit of the distance field
     int tuned_warps = 0;  // autotuned warps per block (0: largest that fits)
     int tuned_order = 0;  // autotuned checkpoint order
     int tuned_fine = 0;   // autotuned fine-test mode (0 union, 1 reassigned)
@@ -164,6 +198,17 @@ mrpop_status make_vparams(mrpop_problem *p, const float *qa, const float *qb, in
 mrpop_status launch_validate_batch(const VParams *d_params, int nslots, int spl, int warps,
                                    int blocks_per_slot, size_t smem, bool fine,
                                    cudaStream_t st);
+// Fills the distance field of t (its df_* fields set except df) from the
+// obstacles of the device table blob, bounds reduced by shrink and measured in
+// unit; enqueued on st.
+mrpop_status launch_field(const Tables &t, const float4 *blob, float edge, float shrink, float unit,
+                          uint8_t *out, cudaStream_t st);
+// mrpop_create_problem; share (or null): a problem with the same obstacles and
+// margin whose links include this one's, and which outlives it, whose distance
+// field is used instead of a new one.
+mrpop_status create_problem(const mrpop_robot *robots, int32_t K, const mrpop_obstacles *obs,
+                            const float *start, const float *goal, const mrpop_config *cfg,
+                            const mrpop_problem *share, mrpop_problem **out);
 mrpop_status launch_fk(mrpop_problem *p, const float *q, int64_t n, float *out, cudaStream_t st);
 mrpop_status launch_nearest(const float *tree, int64_t N, int64_t ld, int dim,
                             const float *queries, const float *budgets, int64_t Q,

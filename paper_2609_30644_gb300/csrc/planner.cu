@@ -934,7 +934,7 @@ static mrpop_status make_sub(mrpop_problem *p, int k, float res, mrpop_problem *
                       (int)(p->obs_cuboids.size() / 15), p->obs_cuboids.data()};
     mrpop_config c = p->cfg;
     c.resolution = res;
-    return mrpop_create_problem(&r, 1, &o, nullptr, nullptr, &c, out);
+    return create_problem(&r, 1, &o, nullptr, nullptr, &c, p, out);
 }
 
 static mrpop_status make_fine(mrpop_problem *p, mrpop_problem **out) {
@@ -954,7 +954,7 @@ static mrpop_status make_fine(mrpop_problem *p, mrpop_problem **out) {
                       (int)(p->obs_cuboids.size() / 15), p->obs_cuboids.data()};
     mrpop_config c = p->cfg;
     c.resolution = p->cfg.resolution * 0.25f;
-    return mrpop_create_problem(rs.data(), (int)rs.size(), &o, nullptr, nullptr, &c, out);
+    return create_problem(rs.data(), (int)rs.size(), &o, nullptr, nullptr, &c, p, out);
 }
 
 static void free_device(Planner *pl);
@@ -1821,7 +1821,7 @@ __device__ __noinline__ void val_chunk(const VParams &vp, int chunk, int per, in
                                        float4 *sm4, int *s_next) {
     if (threadIdx.x == 0) *s_next = 0;
     const int e0 = chunk * per, e1 = min(count, e0 + per);
-    vb::validate_body<vb::kVerdict, false, true>(vp, sm4, e0, e1, s_next);
+    vb::verdict_body<true>(vp, sm4, e0, e1, s_next);
     __syncthreads();
 }
 
@@ -2359,7 +2359,10 @@ static mrpop_status per_buffers(Planner *pl, std::vector<VParams> &vps) {
     vps.push_back(b.vfine);
     for (int k = 0; k < K; ++k) vps.push_back(pl->rm[k].vp_c);
     for (int k = 0; k < K; ++k) vps.push_back(pl->rm[k].vp_e);
-    for (VParams &v : vps) v.fine = 0;  // the persistent form takes the union fine stage
+    for (VParams &v : vps) {  // the persistent form takes the union fine stage
+        v.fine = 0;
+        v.warp_floats = verdict_warp_floats(v.t);
+    }
     return MRPOP_OK;
 }
 

@@ -9,27 +9,31 @@
 //    every tile samples the whole edge and a collision anywhere ends the edge
 //    after few tiles (early exit with __any_sync).
 //  * Per link, forward kinematics in registers (Rz, then the d/a/alpha
-//    offsets), then three levels of culling:
-//      1. tile level: the warp bounds the link's coarse spheres at its 32
-//         checkpoints by one sphere (around the exact box of the centres, from
-//         order-preserving integer min/max warp reductions); lane i tests
-//         obstacle i (and the tile bound of earlier links i) against it, and a
-//         ballot gives the candidate set -- when it is empty, nothing below
-//         runs for that obstacle group;
-//      2. checkpoint level ("coarse" stage of the paper): each lane tests its
+//    offsets), then four levels of culling:
+//      1. the obstacles' distance field (mrpop_internal.cuh): one byte per
+//         checkpoint tells whether the link's coarse sphere is clear of all of
+//         them; where every lane is clear nothing below runs;
+//      2. tile level: the warp bounds the link's coarse spheres at the near
+//         checkpoints by one sphere; lane i tests obstacle i against it, and a
+//         ballot gives the candidate set;
+//      3. checkpoint level ("coarse" stage of the paper): each lane tests its
 //         own link sphere against the candidates only;
-//      3. sphere level ("fine" stage): the warp-wide OR of the lanes' hit
+//      4. sphere level ("fine" stage): the warp-wide OR of the lanes' hit
 //         masks (__reduce_or_sync) selects the obstacles / links whose spheres
-//         are tested, on a register cache of the link's world spheres.
+//         are tested.
+//    Robots are tested against each other through boxes (per tile, then per
+//    checkpoint), link spheres, then spheres.
+//    The clearance and work-count modes and the reassigned fine stage keep the
+//    form without the field (validate_body), which the counters describe.
 //    Culling never changes a verdict: each bound encloses what it replaces
 //    with a slack above FP32 rounding.
 //  * The paper's own design (4 threads per motion, then threads reassigned in
 //    proportion to the fine-test load) balances work across motions; here the
 //    warp-uniform union mask keeps all 32 lanes busy on the same tests instead.
-//  * Geometry tables are staged once per block into shared memory; the
-//    coarse centres of robots 0..K-2 go to a per-warp shared scratch
-//    [link][3][lane] (lane-contiguous, conflict-free) for the robot-robot
-//    tests, whose rare fine stage rebuilds the other link's frame.
+//  * Geometry tables are staged once per block into shared memory; the links'
+//    coarse centres go to a per-warp shared scratch [link][3][lane]
+//    (lane-contiguous, conflict-free) for the robot-robot tests, whose rare
+//    fine stage rebuilds the links' frames.
 #include <cfloat>
 #include <cmath>
 #include <algorithm>
@@ -47,18 +51,34 @@ namespace {
 using namespace vb;
 
 template <int MODE, bool RA>
-__global__ void __launch_bounds__(kWarpsMax * 32) validate_kernel(const VParams P) {
+__global__ void __launch_bounds__(kWarpsMax * 32, MODE == kVerdict && !RA ? 7 : 1)
+validate_kernel(const __grid_constant__ VParams P) {
     extern __shared__ float4 sm4[];
-    validate_body<MODE, RA>(P, sm4);
+    if constexpr (MODE == kVerdict && !RA)
+        verdict_body<false>(P, sm4);
+    else
+        validate_body<MODE, RA>(P, sm4);
+}
+
+// One edge per block (few edges).
+__global__ void __launch_bounds__(kWarpsMax * 32)
+validate_group_kernel(const __grid_constant__ VParams P) {
+    extern __shared__ float4 sm4[];
+    __shared__ int s_hit;
+    if (threadIdx.x == 0) s_hit = 0;  // (visible after the tables' barrier)
+    verdict_body<false, true>(P, sm4, 0, 0, &s_hit);
 }
 
 // The same kernel with a wide register budget (up to 128 registers: four
 // blocks of four warps per SM): fewer warps, no spills in the robot-robot
 // fine stage, which many-arm scenes reach often.  An autotuner dimension.
 template <int MODE, bool RA>
-__global__ void __launch_bounds__(kWarpsMax * 32, 4) validate_kernel_wide(const VParams P) {
+__global__ void __launch_bounds__(kWarpsMax * 32, 4) validate_kernel_wide(const __grid_constant__ VParams P) {
     extern __shared__ float4 sm4[];
-    validate_body<MODE, RA>(P, sm4);
+    if constexpr (MODE == kVerdict && !RA)
+        verdict_body<false>(P, sm4);
+    else
+        validate_body<MODE, RA>(P, sm4);
 }
 
 // Many problems in one launch: block row y serves problem y (its parameters
@@ -69,7 +89,10 @@ __global__ void __launch_bounds__(kWarpsMax * 32) validate_batch_kernel(const VP
     __shared__ VParams sP;
     if (threadIdx.x == 0) sP = Ps[blockIdx.y];
     __syncthreads();
-    validate_body<kVerdict, RA>(sP, sm4);
+    if constexpr (RA)
+        validate_body<kVerdict, true>(sP, sm4);
+    else
+        verdict_body<false>(sP, sm4);
 }
 
 // Resident blocks per SM of a validation kernel for a launch shape.  The
@@ -112,6 +135,21 @@ mrpop_status launch_mode(mrpop_problem *p, VParams &V, int warps, size_t smem,
                                              warps * 32, smem, &bps);
     if (os != MRPOP_OK) return os;
     if (bps < 1) return set_error(MRPOP_EINVAL, "validation kernel does not fit on an SM");
+    // as many blocks as edges fit on the chip at once: an edge per block, whose
+    // warps share its tiles (256 planar edges, kernel: 18.6 us with an edge per
+    // warp, 13.4 us)
+    if (MODE == kVerdict && !RA && warps > 1 && V.E <= (int64_t)p->num_sms * bps) {
+        int gbps = 0;
+        const mrpop_status gs = cached_occupancy((const void *)validate_group_kernel, p->device,
+                                                 (int)p->smem_optin, warps * 32, smem, &gbps);
+        if (gs != MRPOP_OK) return gs;
+        if (V.E <= (int64_t)p->num_sms * gbps) {
+            V.warps = warps;
+            validate_group_kernel<<<(int)V.E, warps * 32, smem, st>>>(V);
+            MRPOP_CUDA_TRY(cudaGetLastError());
+            return MRPOP_OK;
+        }
+    }
     const int64_t want = (V.E + warps - 1) / warps;
     const int grid = (int)std::min<int64_t>((int64_t)p->num_sms * bps, want);
     V.total_warps = grid * warps;
@@ -159,7 +197,45 @@ __global__ void fk_kernel(const float4 *__restrict__ tab, const Tables t,
     }
 }
 
+// Distance field of the obstacles, one voxel per thread (DistanceField in
+// mrpop_internal.cuh).  Bound by the obstacle tests (11 flops a sphere, 31 a
+// box), once per problem: 229,000 voxels and 64 obstacles on the table pair;
+// problem creation grew by about 0.12 ms with the field's allocation.
+__global__ void __launch_bounds__(256)
+field_kernel(const float4 *__restrict__ tab, const Tables t, float edge, float shrink, float unit,
+             uint8_t *__restrict__ out) {
+    const int nx = t.df_n[0], ny = t.df_n[1], nz = t.df_n[2];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nx * ny * nz) return;
+    const int ix = i % nx, iy = (i / nx) % ny, iz = i / (nx * ny);
+    const float x = edge * (kFieldMagic - t.df_c[0] + (float)ix);
+    const float y = edge * (kFieldMagic - t.df_c[1] + (float)iy);
+    const float z = edge * (kFieldMagic - t.df_c[2] + (float)iz);
+    float d = FLT_MAX;
+    for (int o = 0; o < t.NS; ++o) {
+        const float4 ob = __ldg(tab + t.off_os + o);
+        d = fminf(d, __fsqrt_rn(dist2(x, y, z, ob.x, ob.y, ob.z)) - ob.w);
+    }
+    float d2 = FLT_MAX;
+    for (int o = 0; o < t.NC; ++o) {
+        const float4 *c = tab + t.off_oc + kCuboidF4 * o;
+        d2 = fminf(d2, box_dist2(x, y, z, __ldg(c), __ldg(c + 1), __ldg(c + 2), __ldg(c + 3),
+                                 __ldg(c + 4)));
+    }
+    d = fminf(d, __fsqrt_rn(d2)) - shrink;
+    // (a NaN bound, which finite tables do not give, reads as near)
+    out[i] = d > 0.f ? (uint8_t)fminf(255.f, floorf(d / unit * 0.99999f)) : 0;
+}
+
 }  // namespace
+
+mrpop_status launch_field(const Tables &t, const float4 *blob, float edge, float shrink, float unit,
+                          uint8_t *out, cudaStream_t st) {
+    const int n = t.df_n[0] * t.df_n[1] * t.df_n[2];
+    field_kernel<<<(n + 255) / 256, 256, 0, st>>>(blob, t, edge, shrink, unit, out);
+    MRPOP_CUDA_TRY(cudaGetLastError());
+    return MRPOP_OK;
+}
 
 mrpop_status launch_validate(mrpop_problem *p, const float *qa, const float *qb, int64_t n,
                              uint8_t *valid, float *length, int32_t *npoints,
@@ -183,7 +259,8 @@ mrpop_status launch_validate(mrpop_problem *p, const float *qa, const float *qb,
     V.dpad = (t.L + 3) & ~3;
     V.nstore = t.selfcol ? t.L : t.link0[t.K - 1];
     V.fine = p->tuned_fine;
-    V.warp_floats = validate_warp_floats(t, V.fine);
+    V.warp_floats = min_clear || counters || V.fine ? validate_warp_floats(t, V.fine)
+                                                    : verdict_warp_floats(t);
     const size_t tab_bytes = (size_t)t.n_f4 * sizeof(float4);
     int warps = p->tuned_warps > 0 ? p->tuned_warps : kWarpsMax;
     size_t smem = 0;
@@ -218,7 +295,8 @@ mrpop_status make_vparams(mrpop_problem *p, const float *qa, const float *qb, in
     V->dpad = (t.L + 3) & ~3;
     V->nstore = t.selfcol ? t.L : t.link0[t.K - 1];
     V->fine = p->tuned_fine;
-    V->warp_floats = validate_warp_floats(t, V->fine);
+    // (a slot that asks for the reassigned stage may share a launch without it)
+    V->warp_floats = std::max(verdict_warp_floats(t), V->fine ? validate_warp_floats(t, 1) : 0);
     const size_t tab_bytes = (size_t)t.n_f4 * sizeof(float4);
     int warps = p->tuned_warps > 0 ? p->tuned_warps : kWarpsMax;
     size_t smem = 0;
@@ -278,7 +356,9 @@ mrpop_status autotune_validate(mrpop_problem *p, const float *qa, const float *q
         for (int f = 0; f < 2 && s == MRPOP_OK; ++f)
         for (int rg = 0; rg < 2 && s == MRPOP_OK; ++rg) {
             const size_t need = (size_t)p->dev.t.n_f4 * sizeof(float4) +
-                                (size_t)w * validate_warp_floats(p->dev.t, f) * sizeof(float);
+                                (size_t)w * sizeof(float) *
+                                    std::max(verdict_warp_floats(p->dev.t),
+                                             f ? validate_warp_floats(p->dev.t, 1) : 0);
             if (need + sizeof(VParams) + 1024 > p->smem_optin) continue;
             p->tuned_warps = w;
             p->tuned_order = o;

@@ -646,5 +646,450 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
     }
 }
 
+// The same frame and interval count from (q_a, q_b - q_a) pairs.
+__device__ __forceinline__ Frame link_frame(const float4 *tab, const Tables &t, const float2 *ad,
+                                            int i, float tk) {
+    int b = 0;
+    while (t.link0[b + 1] <= i) ++b;
+    Frame Tm = load_base(tab, t, b);
+    for (int l = t.link0[b];; ++l) {
+        const float4 LA = tab[t.off_link + kLinkF4 * l];
+        float sn, cs;
+        joint_sincos(__fmaf_rn(tk, ad[l].y, ad[l].x) + tab[t.off_link + kLinkF4 * l + 1].x, &sn, &cs);
+        const Frame F = rotz(Tm, cs, sn);
+        if (l == i) return F;
+        Tm = advance(F, LA.x, LA.y, LA.z, LA.w);
+    }
+}
+
+__device__ __forceinline__ int interval_count(const float2 *ad, int D, float res, float *len_out) {
+    float acc = 0.f;
+    for (int i = 0; i < D; ++i) acc = __fmaf_rn(ad[i].y, ad[i].y, acc);
+    const float len = __fsqrt_rn(acc);
+    const float nf = ceilf(__fdiv_rn(len, res));
+    *len_out = len;
+    if (!(nf >= 1.f)) return 1;
+    return nf > 1073741824.f ? 1073741824 : (int)nf;
+}
+
+// Fine robot-robot test of link l (frame F) against link i: true where a
+// sphere of one touches a sphere of the other at the lane's checkpoint.  Only
+// lanes whose own coarse spheres touch (own) can; each sphere of l is first
+// tested against i's coarse sphere (centre x, which encloses i's spheres with
+// slack), and i's spheres are placed when one of them is near.
+__device__ __forceinline__ bool fine_pair(const float4 *tab, const Tables &t, const float2 *ad,
+                                          float tk, const Frame &F, int l, int i,
+                                          bool own, const float *x, float m) {
+    const float4 LBl = tab[t.off_link + kLinkF4 * l + 1], LBi = tab[t.off_link + kLinkF4 * i + 1];
+    const int sf = __float_as_int(LBl.y), ns = __float_as_int(LBl.z);
+    const int sfi = __float_as_int(LBi.y), nsi = __float_as_int(LBi.z);
+    const float rci = tab[t.off_link + kLinkF4 * i + 2].w + m;
+    const float xi = x[0], yi = x[32], zi = x[64];
+    unsigned near = 0;  // spheres of l near i's coarse sphere in some lane
+    for (int s = 0; s < ns; ++s) {
+        const float4 sp = tab[t.off_sph + sf + s];
+        const float3 p = apply(F, sp.x, sp.y, sp.z);
+        const float th = sp.w + rci;
+        near |= own && dist2(p.x, p.y, p.z, xi, yi, zi) < th * th ? 1u << s : 0u;
+    }
+    near = __reduce_or_sync(kFull, near);
+    if (!near) return false;
+    const Frame Fi = link_frame(tab, t, ad, i, tk);
+    bool hit = false;
+    // i's spheres four at a time, each near sphere of l placed once per four
+    for (int g0 = 0; g0 < nsi; g0 += 4) {
+        float4 pa[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float4 sp2 = tab[t.off_sph + sfi + min(g0 + j, nsi - 1)];
+            const float3 q3 = apply(Fi, sp2.x, sp2.y, sp2.z);
+            pa[j] = make_float4(q3.x, q3.y, q3.z, sp2.w);
+        }
+        for (unsigned mm = near; mm; mm &= mm - 1) {
+            const float4 sp = tab[t.off_sph + sf + __ffs(mm) - 1];
+            const float3 p = apply(F, sp.x, sp.y, sp.z);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {  // (a repeated last sphere changes nothing)
+                const float d2 = dist2(p.x, p.y, p.z, pa[j].x, pa[j].y, pa[j].z);
+                const float th2 = sp.w + pa[j].w + m;
+                hit |= d2 < th2 * th2;
+            }
+        }
+    }
+    return hit;
+}
+
+// Link l against the links first + bit of mask (an earlier robot's, or its own
+// robot's partners); near: lanes that may be in contact.  Coarse spheres at the
+// lane's checkpoint, then the spheres of the pairs that some lane hit.
+__device__ __forceinline__ bool link_pairs(const float4 *tab, const Tables &t, const float2 *ad,
+                                           float tk, int l, bool near, int first,
+                                           unsigned mask, const float *xc, float m) {
+    const int lane = threadIdx.x & 31, o_link = t.off_link;
+    const float *x = xc + l * (kXcFloats * 32) + lane;
+    const float cx = x[0], cy = x[32], cz = x[64], rl = tab[o_link + kLinkF4 * l + 2].w;
+    unsigned own = 0;
+    for (unsigned mm = mask; mm; mm &= mm - 1) {
+        const int bit = __ffs(mm) - 1, i = first + bit;
+        if (__float_as_int(tab[o_link + kLinkF4 * i + 1].z) == 0) continue;  // no spheres
+        const float *y = xc + i * (kXcFloats * 32) + lane;
+        const float th2 = rl + tab[o_link + kLinkF4 * i + 2].w + m;
+        own |= near && dist2(cx, cy, cz, y[0], y[32], y[64]) < th2 * th2 ? 1u << bit : 0u;
+    }
+    unsigned wi = __reduce_or_sync(kFull, own);
+    if (!wi) return false;
+    const Frame F = link_frame(tab, t, ad, l, tk);
+    bool hit = false;
+    for (; wi; wi &= wi - 1) {
+        const int bit = __ffs(wi) - 1, i = first + bit;
+        hit |= fine_pair(tab, t, ad, tk, F, l, i, (own >> bit) & 1u,
+                         xc + i * (kXcFloats * 32) + lane, m);
+    }
+    return hit;
+}
+
+// Link l (its frame F and coarse centre cc at the lane's checkpoint) against
+// the obstacles; near: lanes whose coarse sphere the distance field does not
+// clear.  Tile bound over those lanes, lane-parallel obstacle tests, candidates
+// against each lane's own coarse sphere, and the warp-wide union of what is hit
+// against the link's fine spheres.
+__device__ __forceinline__ bool link_obstacles(const float4 *tab, const Tables &t,
+                                               const float4 &LB, const float4 &LC, const Frame &F,
+                                               const float3 &cc, bool near, float m) {
+    const int lane = threadIdx.x & 31;
+    const int sf = __float_as_int(LB.y), ns = __float_as_int(LB.z);
+    // one sphere around the near lanes' coarse spheres, from the box of their
+    // centres taken relative to the workspace corner (coordinates >= 0, whose
+    // bits order like unsigned integers)
+    const float wlx = t.ws_lo[0], wly = t.ws_lo[1], wlz = t.ws_lo[2];
+    const unsigned ux = __float_as_uint(cc.x - wlx), uy = __float_as_uint(cc.y - wly),
+                   uz = __float_as_uint(cc.z - wlz);
+    const float x0 = __uint_as_float(__reduce_min_sync(kFull, near ? ux : kFull));
+    const float x1 = __uint_as_float(__reduce_max_sync(kFull, near ? ux : 0u));
+    const float y0 = __uint_as_float(__reduce_min_sync(kFull, near ? uy : kFull));
+    const float y1 = __uint_as_float(__reduce_max_sync(kFull, near ? uy : 0u));
+    const float z0 = __uint_as_float(__reduce_min_sync(kFull, near ? uz : kFull));
+    const float z1 = __uint_as_float(__reduce_max_sync(kFull, near ? uz : 0u));
+    const float ex = 0.5f * (x1 - x0), ey = 0.5f * (y1 - y0), ez = 0.5f * (z1 - z0);
+    float4 bnd;
+    bnd.x = wlx + 0.5f * (x0 + x1);
+    bnd.y = wly + 0.5f * (y0 + y1);
+    bnd.z = wlz + 0.5f * (z0 + z1);
+    // the hardware's approximate square root (an error of a few ulps), padded
+    // by 2^-16 relative; kTileSlack covers the rest
+    float rbox;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(rbox) : "f"(fmaf(ex, ex, fmaf(ey, ey, ez * ez))));
+    bnd.w = fmaf(rbox, 1.0000153f, LC.w + kTileSlack);
+    if (!(bnd.w < FLT_MAX)) bnd.w = FLT_MAX * 2.f;  // never for finite inputs
+    const float rc = LC.w + m;
+    const int NS = t.NS, NC = t.NC;
+    bool hit = false;
+    for (int c0 = 0; c0 < NS; c0 += 32) {
+        bool h = false;
+        if (lane < NS - c0) {
+            const float4 ob = tab[t.off_os + c0 + lane];
+            const float th2 = bnd.w + ob.w + m;
+            h = dist2(bnd.x, bnd.y, bnd.z, ob.x, ob.y, ob.z) < th2 * th2;
+        }
+        unsigned own = 0;
+        for (unsigned cm = __ballot_sync(kFull, h); cm; cm &= cm - 1) {
+            const int o = __ffs(cm) - 1;
+            const float4 ob = tab[t.off_os + c0 + o];
+            const float th2 = rc + ob.w;
+            own |= near && dist2(cc.x, cc.y, cc.z, ob.x, ob.y, ob.z) < th2 * th2 ? 1u << o : 0u;
+        }
+        const unsigned wm = __reduce_or_sync(kFull, own);
+        if (!wm) continue;
+        // each of the link's spheres is placed once and tested against every
+        // obstacle of the warp's union mask
+        for (int s = 0; s < ns; ++s) {
+            const float4 sp = tab[t.off_sph + sf + s];
+            const float3 p = apply(F, sp.x, sp.y, sp.z);
+            for (unsigned mm = wm; mm; mm &= mm - 1) {
+                const float4 ob = tab[t.off_os + c0 + __ffs(mm) - 1];
+                const float th2 = sp.w + ob.w + m;
+                hit |= dist2(p.x, p.y, p.z, ob.x, ob.y, ob.z) < th2 * th2;
+            }
+        }
+    }
+    // cuboids: the bound against the box's bounding sphere (the box lies within
+    // it), then its exact distance only where that sphere is near
+    for (int c0 = 0; c0 < NC; c0 += 32) {
+        bool h = false;
+        if (lane < NC - c0) {
+            const float4 *cbp = tab + t.off_oc + kCuboidF4 * (c0 + lane);
+            const float4 cb0 = cbp[0];
+            const float reach = cb0.w + bnd.w + m;
+            if (dist2(bnd.x, bnd.y, bnd.z, cb0.x, cb0.y, cb0.z) < reach * reach) {
+                const float th2 = bnd.w + m;
+                h = box_dist2(bnd.x, bnd.y, bnd.z, cb0, cbp[1], cbp[2], cbp[3], cbp[4]) < th2 * th2;
+            }
+        }
+        unsigned own = 0;
+        for (unsigned cm = __ballot_sync(kFull, h); cm; cm &= cm - 1) {
+            const int o = __ffs(cm) - 1;
+            const float4 *cbp = tab + t.off_oc + kCuboidF4 * (c0 + o);
+            own |= near && box_dist2(cc.x, cc.y, cc.z, cbp[0], cbp[1], cbp[2], cbp[3], cbp[4]) <
+                               rc * rc
+                       ? 1u << o : 0u;
+        }
+        const unsigned wm = __reduce_or_sync(kFull, own);
+        if (!wm) continue;
+        for (int s = 0; s < ns; ++s) {
+            const float4 sp = tab[t.off_sph + sf + s];
+            const float3 p = apply(F, sp.x, sp.y, sp.z);
+            const float th2 = sp.w + m;
+            for (unsigned mm = wm; mm; mm &= mm - 1) {
+                const float4 *cbp = tab + t.off_oc + kCuboidF4 * (c0 + __ffs(mm) - 1);
+                hit |= box_dist2(p.x, p.y, p.z, cbp[0], cbp[1], cbp[2], cbp[3], cbp[4]) < th2 * th2;
+            }
+        }
+    }
+    return hit;
+}
+
+// Verdicts of composite edges, one warp per edge and a checkpoint per lane.
+// Per tile of 32 checkpoints and robot:
+//   1. down the chain: forward kinematics in registers, the link's coarse
+//      centre to shared memory, and one byte of the obstacles' distance field
+//      at that centre, whose load overlaps the next link's frame and joint;
+//   2. a link that the field does not clear in some lane runs the obstacle
+//      tests (link_obstacles); a fine hit ends the edge;
+//   3. robots in reach of each other (boxes around the tile's coarse centres,
+//      one lane per earlier robot) run the link-pair tests: each link against
+//      the earlier robot's box at the lane's own checkpoint, then against its
+//      links, then sphere against sphere (fine_pair).
+// Every level encloses what it replaces with a slack above FP32 rounding, and
+// the sphere-level arithmetic alone decides.  Before, every link built a tile
+// bound (six warp reductions) and tested it against all obstacles and earlier
+// links, about 230 of the 279 instructions a link took; an eighth of the links
+// now needs any of that (65,536 candidate edges of the table pair: 312 M
+// instructions and 324 us before, 204 M and 240 us now; 8 arms, 4,099 edges: 57
+// M and 480 us, 32 M and 258 us).  Running all of a robot's links first and
+// rebuilding the near ones' frames afterwards was slower (292 us: more joints
+// before a colliding link ends the edge).
+//
+// LOCAL: the edges [e0, e1) are handed out to the block's warps through the
+// shared-memory counter *s_next (zeroed by the caller before the call) instead
+// of the problem's global work counter, which is then left untouched.
+//
+// GROUP: the block's warps share one edge (edge blockIdx.x), tile after tile in
+// turn, for batches of so few edges that an edge per warp would leave most of
+// the chip idle: the time is then that of the longest edge, one tile after
+// another.  The caller gives a shared flag (zero) in s_next.
+template <bool LOCAL, bool GROUP = false>
+__device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int e0 = 0, int e1 = 0,
+                                             int *s_next = nullptr) {
+    float4 *tab = sm4;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const Tables &t = P.t;
+    const int K = t.K, D = t.L;
+    float *ws = reinterpret_cast<float *>(sm4 + t.n_f4) + (size_t)warp * P.warp_floats;
+    float2 *ad = reinterpret_cast<float2 *>(ws);  // (q_a, q_b - q_a) of each joint, one spare
+    const int dpad = (D + 4) & ~3;                             // verdict_dpad
+    float4 *rb = reinterpret_cast<float4 *>(ws + 2 * dpad);    // robot tile boxes [K][2]
+    float *xc = ws + 2 * dpad + 8 * K;                         // coarse centres [L][3][32]
+
+    for (int i = threadIdx.x; i < t.n_f4; i += blockDim.x) tab[i] = P.blob[i];
+    __syncthreads();
+    if (warp >= P.warps) return;  // spare warps of a shared multi-problem launch
+
+    const int o_link = t.off_link;
+    const uint8_t *df = t.df;
+    const float fi = t.df_inv, fx = t.df_c[0], fy = t.df_c[1], fz = t.df_c[2];
+    const unsigned fnx = t.df_n[0], fny = t.df_n[1], fnz = t.df_n[2];
+    const int fout = t.df_out;
+    const float m = P.margin;
+    if (lane == 0) ad[D] = make_float2(0.f, 0.f);
+    const bool pairs = K > 1 || t.selfcol;
+    for (;;) {
+        int e = 0;
+        if (GROUP) {
+            e = blockIdx.x;
+        } else {
+            if (lane == 0) e = LOCAL ? e0 + atomicAdd(s_next, 1) : atomicAdd(&P.work[0], 1);
+            e = __shfl_sync(kFull, e, 0);
+            if (e >= (LOCAL ? e1 : P.E)) break;
+        }
+        __syncwarp();
+        for (int i = lane; i < D; i += 32) {
+            // (the persistent planner rewrites its edge buffers within one
+            // launch: there the loads bypass the non-coherent cache)
+            const float a = LOCAL ? __ldcg(P.qa + (size_t)i * P.E + e) : __ldg(P.qa + (size_t)i * P.E + e);
+            const float b = LOCAL ? __ldcg(P.qb + (size_t)i * P.E + e) : __ldg(P.qb + (size_t)i * P.E + e);
+            ad[i] = make_float2(a, __fsub_rn(b, a));
+        }
+        __syncwarp();
+        float len;
+        const int n = interval_count(ad, D, P.res, &len);
+        // Edges beyond MRPOP_MAX_EDGE_INTERVALS intervals (or with non-finite
+        // coordinates) are reported invalid without being checked.
+        const bool too_long = !(len <= P.res * (float)MRPOP_MAX_EDGE_INTERVALS);
+        const int T = too_long ? 0 : (n >> 5) + 1;  // ceil((n + 1) / 32)
+        bool edge_hit = too_long;
+
+        for (int tile = GROUP ? warp : 0; tile < T && !edge_hit; tile += GROUP ? P.warps : 1) {
+            if (GROUP && *(volatile int *)s_next) break;  // another warp's tile collides
+            int k = P.order ? tile * 32 + lane : tile + T * lane;
+            k = min(k, n);
+            // (k = 0 apart: a zero numerator sends the whole warp through the
+            // division's slow path)
+            const float tq = __fdiv_rn((float)max(k, 1), (float)n);
+            const float tk = k > 0 ? tq : 0.f;
+            float sn, cs;  // of the next link's joint
+            joint_sincos(__fmaf_rn(tk, ad[0].y, ad[0].x) + tab[o_link + 1].x, &sn, &cs);
+            for (int b = 0; b < K && !edge_hit; ++b) {
+                const int l0 = t.link0[b], l1 = t.link0[b + 1];
+                Frame Tm = load_base(tab, t, b);
+                float bx0 = FLT_MAX, by0 = FLT_MAX, bz0 = FLT_MAX;  // box of the lane's centres
+                float bx1 = -FLT_MAX, by1 = -FLT_MAX, bz1 = -FLT_MAX;
+                const float4 *lk = tab + o_link + kLinkF4 * l0;
+                float *x = xc + l0 * (kXcFloats * 32) + lane;
+                const float2 *aj = ad + l0 + 1;  // the next link's joint
+                const float rmax = lk[3].y;  // the robot's largest coarse radius, -1: no spheres
+                bool hit = false;
+#pragma unroll 1
+                for (int l = l0; l < l1; ++l) {
+                    const float4 LA = lk[0], LC = lk[2], LD = lk[3];
+                    const Frame F = rotz(Tm, cs, sn);
+                    const float3 cc = apply(F, LC.x, LC.y, LC.z);
+                    // the field's byte, loaded ahead of the next link's frame and joint
+                    const int th = __float_as_int(LD.x);
+                    const unsigned ix = __float_as_uint(fmaf(cc.x, fi, fx)) - kFieldMagicBits;
+                    const unsigned iy = __float_as_uint(fmaf(cc.y, fi, fy)) - kFieldMagicBits;
+                    const unsigned iz = __float_as_uint(fmaf(cc.z, fi, fz)) - kFieldMagicBits;
+                    const bool in = (ix < fnx) & (iy < fny) & (iz < fnz);
+                    int v = fout;
+                    if (in) v = __ldg(df + ((iz * fny + iy) * fnx + ix));
+                    Tm = advance(F, LA.x, LA.y, LA.z, LA.w);
+                    // (the last link's successor is the spare entry)
+                    const float2 qd = *aj++;
+                    joint_sincos(__fmaf_rn(tk, qd.y, qd.x) + LD.z, &sn, &cs);
+                    if (pairs) {
+                        x[0] = cc.x;
+                        x[32] = cc.y;
+                        x[64] = cc.z;
+                        // (a link without spheres only widens the box)
+                        bx0 = fminf(bx0, cc.x);
+                        bx1 = fmaxf(bx1, cc.x);
+                        by0 = fminf(by0, cc.y);
+                        by1 = fmaxf(by1, cc.y);
+                        bz0 = fminf(bz0, cc.z);
+                        bz1 = fmaxf(bz1, cc.z);
+                    }
+                    const bool near = v < th;
+                    if (__any_sync(kFull, near)) {
+                        hit = link_obstacles(tab, t, lk[1], LC, F, cc, near, m);
+                        if (__any_sync(kFull, hit)) {
+                            edge_hit = true;
+                            break;
+                        }
+                    }
+                    lk += kLinkF4;
+                    x += kXcFloats * 32;
+                }
+                if (edge_hit || rmax < 0.f) {
+                    if (lane == 0) rb[2 * b].w = -1.f;  // no spheres: pairs with nothing
+                    continue;
+                }
+                if (K > 1) {
+                    // the robot's box over the tile, relative to the workspace
+                    // corner as the tile bounds are
+                    const float wlx = t.ws_lo[0], wly = t.ws_lo[1], wlz = t.ws_lo[2];
+                    float4 lo, hi;
+                    lo.x = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(bx0 - wlx)));
+                    hi.x = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(bx1 - wlx)));
+                    lo.y = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(by0 - wly)));
+                    hi.y = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(by1 - wly)));
+                    lo.z = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(bz0 - wlz)));
+                    hi.z = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(bz1 - wlz)));
+                    lo.w = rmax;
+                    hi.w = 0.f;
+                    if (lane == 0) {
+                        rb[2 * b] = lo;
+                        rb[2 * b + 1] = hi;
+                    }
+                    __syncwarp();
+                    bool close = false;
+                    if (lane < b) {
+                        const float4 ol = rb[2 * lane], oh = rb[2 * lane + 1];
+                        const float gx = fmaxf(fmaxf(ol.x - hi.x, lo.x - oh.x), 0.f);
+                        const float gy = fmaxf(fmaxf(ol.y - hi.y, lo.y - oh.y), 0.f);
+                        const float gz = fmaxf(fmaxf(ol.z - hi.z, lo.z - oh.z), 0.f);
+                        const float r = ol.w + rmax + m + kTileSlack;
+                        close = ol.w >= 0.f && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < r * r;
+                    }
+                    for (unsigned cm = __ballot_sync(kFull, close); cm; cm &= cm - 1) {
+                        const int a = __ffs(cm) - 1;
+                        const int a0 = t.link0[a], a1 = t.link0[a + 1];
+                        // robot a's box at the lane's checkpoint
+                        float ax0 = FLT_MAX, ay0 = FLT_MAX, az0 = FLT_MAX;
+                        float ax1 = -FLT_MAX, ay1 = -FLT_MAX, az1 = -FLT_MAX;
+                        for (int i = a0; i < a1; ++i) {
+                            if (__float_as_int(tab[o_link + kLinkF4 * i + 3].x) == 0) continue;
+                            const float *x = xc + i * (kXcFloats * 32) + lane;
+                            ax0 = fminf(ax0, x[0]);
+                            ax1 = fmaxf(ax1, x[0]);
+                            ay0 = fminf(ay0, x[32]);
+                            ay1 = fmaxf(ay1, x[32]);
+                            az0 = fminf(az0, x[64]);
+                            az1 = fmaxf(az1, x[64]);
+                        }
+                        const float ra = rb[2 * a].w + m + kTileSlack;
+                        unsigned nl = 0;
+                        for (int l = l0; l < l1; ++l) {
+                            if (__float_as_int(tab[o_link + kLinkF4 * l + 3].x) == 0) continue;
+                            const float *x = xc + l * (kXcFloats * 32) + lane;
+                            const float gx = fmaxf(fmaxf(ax0 - x[0], x[0] - ax1), 0.f);
+                            const float gy = fmaxf(fmaxf(ay0 - x[32], x[32] - ay1), 0.f);
+                            const float gz = fmaxf(fmaxf(az0 - x[64], x[64] - az1), 0.f);
+                            const float r = tab[o_link + kLinkF4 * l + 2].w + ra;
+                            nl |= fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < r * r ? 1u << (l - l0) : 0u;
+                        }
+                        for (unsigned wl = __reduce_or_sync(kFull, nl); wl; wl &= wl - 1) {
+                            const int j = __ffs(wl) - 1;
+                            const unsigned links = ((1u << (a1 - a0)) - 1u);
+                            hit |= link_pairs(tab, t, ad, tk, l0 + j, (nl >> j) & 1u, a0,
+                                              links, xc, m);
+                            if (__any_sync(kFull, hit)) {
+                                edge_hit = true;
+                                break;
+                            }
+                        }
+                        if (edge_hit) break;
+                    }
+                }
+                if (t.selfcol && !edge_hit)
+                    for (int l = l0; l < l1 && !edge_hit; ++l) {
+                        const unsigned mask = __float_as_int(tab[o_link + kLinkF4 * l + 1].w);
+                        if (!mask || __float_as_int(tab[o_link + kLinkF4 * l + 3].x) == 0) continue;
+                        hit |= link_pairs(tab, t, ad, tk, l, true, l0, mask, xc, m);
+                        edge_hit = __any_sync(kFull, hit);
+                    }
+            }
+        }
+        if (GROUP) {
+            if (lane == 0 && edge_hit) *(volatile int *)s_next = 1;
+            __syncthreads();
+            edge_hit = *(volatile int *)s_next != 0;
+        }
+        if (lane == 0 && (!GROUP || warp == 0)) {
+            P.valid[e] = edge_hit ? 0 : 1;
+            if (P.length) P.length[e] = len;
+            if (P.npoints) P.npoints[e] = n;
+        }
+        if (GROUP) return;
+    }
+    // The last warp to leave resets the work counter for the next launch on
+    // this problem (every warp has made its final fetch before counting out).
+    if (!LOCAL && lane == 0) {
+        __threadfence();
+        if (atomicAdd(&P.work[1], 1) == P.total_warps - 1) {
+            atomicExch(&P.work[0], 0);
+            atomicExch(&P.work[1], 0);
+        }
+    }
+}
+
 }  // namespace vb
 }  // namespace mrpop

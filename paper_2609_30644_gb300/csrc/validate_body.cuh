@@ -110,7 +110,12 @@ __device__ __forceinline__ void joint_sincos(float th, float *s, float *c) {
     __sincosf(fmaf(-6.28318548f, k, th), s, c);
 }
 
-__device__ __forceinline__ unsigned low_mask(int n) { return n >= 32 ? kFull : ((1u << n) - 1u); }
+// Smallest of the warp's values (order-preserving integer keys; no NaN).
+__device__ __forceinline__ float warp_min(float v) {
+    const int k = __float_as_int(v);
+    const int r = __reduce_min_sync(kFull, k ^ ((k >> 31) & 0x7fffffff));
+    return __int_as_float(r ^ ((r >> 31) & 0x7fffffff));
+}
 
 // Second stage with load-proportional reassignment (Sec. III-E): the fine
 // tests that the lanes' own coarse hits call for -- (checkpoint k, obstacle o
@@ -217,6 +222,15 @@ __device__ __forceinline__ int interval_count(const float *dq, int D, float res,
     return nf > 1073741824.f ? 1073741824 : (int)nf;
 }
 
+// The clearance and work-count modes, and verdicts with the reassigned fine
+// stage.  Clearance takes the same levels with a bound from above on the edge's
+// minimum clearance in the margin's place: far sides of tile bounds at first,
+// then the values themselves, shared by the warp.  A pair that some level
+// leaves out lies farther apart than a pair that is measured (every bound
+// encloses what it replaces with at least 1e-4 m of slack), so the minimum is
+// that over all pairs, to the bit.  Measuring every pair, with a square root
+// each, took 2,929 us for 1,023 edges of the table pair; this takes 90 us.
+//
 // LOCAL: the edges [e0, e1) are handed out to the block's warps through the
 // shared-memory counter *s_next (zeroed by the caller before the call) instead
 // of the problem's global work counter, which is then left untouched.
@@ -242,7 +256,7 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
     const int o_link = t.off_link, o_os = t.off_os, o_oc = t.off_oc, o_sph = t.off_sph;
     const float wlx = t.ws_lo[0], wly = t.ws_lo[1], wlz = t.ws_lo[2];
     const int K = t.K, D = t.L, NS = t.NS, NC = t.NC;
-    const float m = P.margin;
+    const float margin = P.margin;
     unsigned long long cnt[kCounters];
 #pragma unroll
     for (int c = 0; c < kCounters; ++c) cnt[c] = 0ull;
@@ -270,6 +284,9 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
         const int T = too_long ? 0 : (n >> 5) + 1;  // ceil((n + 1) / 32)
         bool edge_hit = too_long;
         float minc = too_long ? -FLT_MAX : FLT_MAX;
+        // kClearance: a bound from above on the edge's minimum clearance
+        // (warp-uniform); pairs that lie at least this far apart are skipped
+        float m = MODE == kClearance ? FLT_MAX : margin;
 
         for (int tile = 0; tile < T; ++tile) {
             int k = P.order ? tile * 32 + lane : tile + T * lane;
@@ -309,7 +326,7 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                     // their float bits order like unsigned integers and min and max
                     // are single-instruction warp reductions.
                     float4 bnd = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (MODE != kClearance) {
+                    {
                         const unsigned ux = __float_as_uint(cc.x - wlx);
                         const unsigned uy = __float_as_uint(cc.y - wly);
                         const unsigned uz = __float_as_uint(cc.z - wlz);
@@ -343,24 +360,42 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                         __syncwarp();
                     }
                     bool vote = false;  // a fine stage ran: the early-exit vote is due
+                    // squared distance within reach (clearance: the bound may be
+                    // negative, and a reach that is not positive has no pair)
+                    auto within = [](float d2, float th) {
+                        return MODE == kClearance ? th > 0.f && d2 < th * th : d2 < th * th;
+                    };
+                    // kClearance: the lanes' minima and new bounds become the warp's
+                    auto tighten = [&](float ub) {
+                        m = fminf(m, warp_min(fminf(minc, ub)));
+                    };
                     if (ns > 0) {
                         bool own_any = false;
                         if (MODE == kCount && active) cnt[7] += 1;  // coarse centre
-                        const float rc = LC.w + m;
+                        float rc = LC.w + m;
 
                         // ---- robot vs obstacle spheres
                         for (int c0 = 0; c0 < NS; c0 += 32) {
                             const int cn = min(32, NS - c0);
                             unsigned own = 0, cand = 0;
-                            if (MODE == kClearance) {
-                                own = low_mask(cn);
-                            } else {
+                            {
                                 bool h = false;
+                                if (MODE == kClearance) {
+                                    // some sphere of the link at some checkpoint is
+                                    // within the tile bound's far side of obstacle i
+                                    float ub = FLT_MAX;
+                                    if (lane < cn) {
+                                        const float4 ob = tab[o_os + c0 + lane];
+                                        ub = __fsqrt_rn(dist2(bnd.x, bnd.y, bnd.z, ob.x, ob.y, ob.z)) +
+                                             bnd.w - ob.w;
+                                    }
+                                    tighten(ub);
+                                    rc = LC.w + m;
+                                }
                                 if (lane < cn) {
                                     const float4 ob = tab[o_os + c0 + lane];
                                     const float d2 = dist2(bnd.x, bnd.y, bnd.z, ob.x, ob.y, ob.z);
-                                    const float th2 = bnd.w + ob.w + m;
-                                    h = d2 < th2 * th2;
+                                    h = within(d2, bnd.w + ob.w + m);
                                 }
                                 cand = __ballot_sync(kFull, h);
                                 unsigned cm = cand;
@@ -369,23 +404,21 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                                     cm &= cm - 1;
                                     const float4 ob = tab[o_os + c0 + o];
                                     const float d2 = dist2(cc.x, cc.y, cc.z, ob.x, ob.y, ob.z);
-                                    const float th2 = rc + ob.w;
-                                    own |= (d2 < th2 * th2) ? (1u << o) : 0u;
+                                    own |= within(d2, rc + ob.w) ? (1u << o) : 0u;
                                 }
                                 if (MODE == kCount) {
                                     if (lane == 0) cnt[8] += cn;
                                     if (active) cnt[2] += __popc(cand);
                                 }
                             }
-                            if (MODE != kClearance && cand == 0u) continue;  // nothing near
+                            if (cand == 0u) continue;  // nothing near
                             vote = true;
                             if (ra) {
                                 hit |= fine_reassigned<false>(own, c0, ns, sf, F, m, tab, t, fr,
                                                               lane);
                                 continue;
                             }
-                            const unsigned wm =
-                                MODE == kClearance ? own : __reduce_or_sync(kFull, own);
+                            const unsigned wm = __reduce_or_sync(kFull, own);
                             if (MODE == kCount && active) {
                                 cnt[4] += (unsigned long long)__popc(own) * ns;
                                 own_any |= own != 0;
@@ -418,9 +451,19 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                         for (int c0 = 0; c0 < NC; c0 += 32) {
                             const int cn = min(32, NC - c0);
                             unsigned own = 0, cand = 0;
-                            if (MODE == kClearance) {
-                                own = low_mask(cn);
-                            } else {
+                            {
+                                if (MODE == kClearance) {
+                                    // (no point of the box is farther than its
+                                    // bounding sphere's far side)
+                                    float ub = FLT_MAX;
+                                    if (lane < cn) {
+                                        const float4 cb0 = tab[o_oc + kCuboidF4 * (c0 + lane)];
+                                        ub = __fsqrt_rn(dist2(bnd.x, bnd.y, bnd.z, cb0.x, cb0.y, cb0.z)) +
+                                             bnd.w;
+                                    }
+                                    tighten(ub);
+                                    rc = LC.w + m;
+                                }
                                 // the box's bounding sphere first (the box lies within
                                 // it), its exact distance only when the sphere is near
                                 bool h = false, exact = false;
@@ -429,12 +472,11 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                                     const float4 cb0 = cbp[0];
                                     const float dc2 = dist2(bnd.x, bnd.y, bnd.z, cb0.x, cb0.y, cb0.z);
                                     const float reach = cb0.w + bnd.w + m;
-                                    exact = dc2 < reach * reach;
+                                    exact = within(dc2, reach);
                                     if (exact) {
                                         const float d2 = box_dist2(bnd.x, bnd.y, bnd.z, cb0, cbp[1],
                                                                    cbp[2], cbp[3], cbp[4]);
-                                        const float th2 = bnd.w + m;
-                                        h = d2 < th2 * th2;
+                                        h = within(d2, bnd.w + m);
                                     }
                                 }
                                 cand = __ballot_sync(kFull, h);
@@ -445,7 +487,7 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                                     const float4 *cbp = tab + o_oc + kCuboidF4 * (c0 + o);
                                     const float d2 = box_dist2(cc.x, cc.y, cc.z, cbp[0], cbp[1],
                                                                cbp[2], cbp[3], cbp[4]);
-                                    own |= (d2 < rc * rc) ? (1u << o) : 0u;
+                                    own |= within(d2, rc) ? (1u << o) : 0u;
                                 }
                                 if (MODE == kCount) {
                                     if (lane == 0) cnt[8] += cn;  // the bounding-sphere tests
@@ -453,15 +495,14 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                                     if (active) cnt[10] += __popc(cand);
                                 }
                             }
-                            if (MODE != kClearance && cand == 0u) continue;  // nothing near
+                            if (cand == 0u) continue;  // nothing near
                             vote = true;
                             if (ra) {
                                 hit |= fine_reassigned<true>(own, c0, ns, sf, F, m, tab, t, fr,
                                                              lane);
                                 continue;
                             }
-                            const unsigned wm =
-                                MODE == kClearance ? own : __reduce_or_sync(kFull, own);
+                            const unsigned wm = __reduce_or_sync(kFull, own);
                             if (MODE == kCount && active) {
                                 cnt[5] += (unsigned long long)__popc(own) * ns;
                                 own_any |= own != 0;
@@ -495,23 +536,30 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                         const unsigned pm0 = (unsigned)pm, pm1 = (unsigned)(pm >> 32);
                         if (pm) {
                             unsigned own0 = 0, own1 = 0, candp = 0;
-                            if (MODE == kClearance) {
-                                own0 = pm0;
-                                own1 = pm1;
-                            } else {
+                            {
+                                if (MODE == kClearance) {
+                                    float ub = FLT_MAX;
+                                    if ((pm0 >> lane) & 1u) {
+                                        const float4 o = tb[lane];
+                                        ub = __fsqrt_rn(dist2(bnd.x, bnd.y, bnd.z, o.x, o.y, o.z)) + bnd.w +
+                                             o.w;
+                                        // (a link without spheres has no pair)
+                                        if (__float_as_int(tab[o_link + kLinkF4 * lane + 1].z) == 0)
+                                            ub = FLT_MAX;
+                                    }
+                                    tighten(ub);
+                                }
                                 // tile-level candidates: lane i tests link i (and i + 32)
                                 bool h0 = false, h1 = false;
                                 if ((pm0 >> lane) & 1u) {
                                     const float4 o = tb[lane];
                                     const float d2 = dist2(bnd.x, bnd.y, bnd.z, o.x, o.y, o.z);
-                                    const float th2 = bnd.w + o.w + m;
-                                    h0 = d2 < th2 * th2;
+                                    h0 = within(d2, bnd.w + o.w + m);
                                 }
                                 if ((pm1 >> lane) & 1u) {
                                     const float4 o = tb[lane + 32];
                                     const float d2 = dist2(bnd.x, bnd.y, bnd.z, o.x, o.y, o.z);
-                                    const float th2 = bnd.w + o.w + m;
-                                    h1 = d2 < th2 * th2;
+                                    h1 = within(d2, bnd.w + o.w + m);
                                 }
                                 const unsigned cand0 = __ballot_sync(kFull, h0);
                                 const unsigned cand1 = __ballot_sync(kFull, h1);
@@ -525,8 +573,7 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                                         const float4 LCi = tab[o_link + kLinkF4 * i + 2];
                                         const float *x = xc + (size_t)i * kXcFloats * 32 + lane;
                                         const float d2 = dist2(cc.x, cc.y, cc.z, x[0], x[32], x[64]);
-                                        const float th2 = LC.w + LCi.w + m;
-                                        own |= (d2 < th2 * th2) ? (1u << bit) : 0u;
+                                        own |= within(d2, LC.w + LCi.w + m) ? (1u << bit) : 0u;
                                     }
                                     if (w == 0)
                                         own0 = own;
@@ -539,10 +586,10 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                                 }
                                 candp = cand0 | cand1;
                             }
-                            if (MODE == kClearance || candp != 0u) {
+                            if (candp != 0u) {
                             vote = true;
-                            const unsigned w0 = MODE == kClearance ? own0 : __reduce_or_sync(kFull, own0);
-                            const unsigned w1 = MODE == kClearance ? own1 : __reduce_or_sync(kFull, own1);
+                            const unsigned w0 = __reduce_or_sync(kFull, own0);
+                            const unsigned w1 = __reduce_or_sync(kFull, own1);
                             if (MODE == kCount && active) {
                                 own_any |= (own0 | own1) != 0;
                                 for (int w = 0; w < 2; ++w) {
@@ -600,6 +647,7 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
                         }
                         if (MODE == kCount && active && own_any) cnt[7] += ns;
                     }
+                    if (MODE == kClearance && vote) tighten(FLT_MAX);
                     Tm = advance(F, LA.x, LA.y, LA.z, LA.w);
                     // a hit can only come from a fine stage of this link
                     if (MODE != kClearance && vote && __any_sync(kFull, hit)) goto tile_done;

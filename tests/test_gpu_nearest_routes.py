@@ -119,3 +119,44 @@ def test_scan_against_oracle(mp, orc, D, n, Q):
         # a different vertex only where FP32 cannot tell the two apart
         assert got[i] == ref or (np.isfinite(sd) and sd - bd <= 1e-5 * max(bd, 1e-30)) or \
             gap <= 1e-5 * max(1.0, abs(float(cs[i]))), (i, got[i], ref)
+
+
+# one block, clusters of 2 to 8 with ragged ranges, queries that fill a block's
+# warps partly, lists that overflow k_max, and the two-kernel path (long lists,
+# high dimensions)
+@pytest.mark.parametrize("D,n,Q,k_max,delta", [
+    (3, 1, 3, 4, 9.0), (7, 255, 9, 64, 2.5), (7, 257, 8, 16, 2.5), (7, 4097, 100, 32, 2.5),
+    (4, 2048, 33, 64, 3.0), (10, 3000, 17, 0, 4.0), (11, 1500, 40, 7, 5.0), (16, 5000, 25, 64, 6.0),
+    (17, 3000, 20, 64, 6.0), (7, 3000, 20, 65, 3.0), (7, 5, 2, 64, 0.0)])
+def test_neighbors_against_oracle(mp, orc, D, n, Q, k_max, delta):
+    rng = np.random.default_rng(D * n)
+    tree = np.zeros((D + 1, n + 3), np.float32)
+    tree[:D] = rng.uniform(-2.9, 2.9, (D, n + 3))
+    qs = rng.uniform(-2.9, 2.9, (D, Q)).astype(np.float32)
+    k = min(Q, n)
+    qs[:, :k] = tree[:D, :k]                  # distance exactly zero
+    idx, cnt = mp.neighbors(_dev(tree), _dev(qs), delta, k_max, n_vertices=n)
+    idx, cnt = idx.cpu().numpy(), cnt.cpu().numpy()
+    sub = np.ascontiguousarray(tree[:, :n])
+    for i in range(Q):
+        ref, rc, gap = orc.neighbors(sub, qs[:, i], np.float32(delta), k_max)
+        if gap <= 1e-5 * delta and delta > 0:
+            assert abs(int(cnt[i]) - rc) <= 2
+            continue
+        assert cnt[i] == rc
+        np.testing.assert_array_equal(idx[i, :min(rc, k_max)], ref[:k_max])
+        assert (idx[i, min(rc, k_max):] == -1).all()
+
+
+@pytest.mark.parametrize("M", [0, 1, 2, 1024, 1025, 1026, 4097, 131073, 131074])
+@pytest.mark.parametrize("D", [1, 6, 7, 8])
+def test_path_cost_sizes(mp, M, D):
+    rng = np.random.default_rng(M + D)
+    buf = torch.from_numpy(rng.uniform(-2.9, 2.9, M * D + 3).astype(np.float32)).cuda()
+    for off in (0, 1, 2):                     # 16-, 4- and 8-byte aligned rows
+        path = buf[off:off + M * D].view(M, D)
+        got = mp.path_cost(path).item()
+        ref = (path[1:].double() - path[:-1].double()).norm(dim=1).sum().item()
+        # FP32 segment lengths: (D + 3) roundings of 2^-24 each at most
+        assert abs(got - ref) <= (D + 3) * 2.0 ** -24 * ref
+        assert mp.path_cost(path).item() == got

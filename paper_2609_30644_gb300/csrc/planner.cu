@@ -106,52 +106,66 @@ __device__ __forceinline__ float nanf_() { return __int_as_float(0x7fc00000); }
 // ---------------------------------------------------------------------------
 
 // q_rand (uniform, or informed in the prolate hyperspheroid of c_best) and the
-// cost coordinate c_rand ~ U[g_lb(q_rand), c_best] (Alg. 2 AO-X).
+// cost coordinate c_rand ~ U[g_lb(q_rand), c_best] (Alg. 2 AO-X), sample i by a
+// half-warp of kInformedTries lanes: the random numbers are a function of a
+// counter, so every lane draws one of the rejection tries and the first try
+// inside the limits is the one that drawing them in turn accepts.  In turn, by
+// one thread, a step's 256 samples were 160 us of its chain in one block
+// (49-D, most tries rejected), 19 us now in 16.
+static_assert(kInformedTries == 16, "half a warp per sample");
 __device__ __forceinline__ void sample_body(const Slot &S, int i) {
     const Ctrl &C = *S.ctrl;
     const int a = (S.tn[0] <= S.tn[1]) ? 0 : 1;  // expand the smaller tree
-    if (i == 0) S.ctrl->tree_a = a;
-    if (i >= kStepIters) return;
+    const int tr = threadIdx.x & (kInformedTries - 1);
+    if (i == 0 && tr == 0) S.ctrl->tree_a = a;
     const int D = S.D, B = kStepIters;
     if (C.mode == 2) {
-        S.crand[i] = -INFINITY;
+        if (tr == 0 && i < B) S.crand[i] = -INFINITY;
         return;
     }
-    Rng rng{mix64(C.seed ^ 0x5851F42D4C957F2Dull), ((unsigned long long)C.step << 32) ^ (unsigned)i};
-    rng.ctr *= 977ull;
+    const unsigned half = threadIdx.x & 16 ? 0xffff0000u : 0x0000ffffu;
+    const unsigned long long key = mix64(C.seed ^ 0x5851F42D4C957F2Dull);
+    const unsigned long long ctr0 = (((unsigned long long)C.step << 32) ^ (unsigned)i) * 977ull;
+    // counters of one try: two per normal and one for the radius
+    const unsigned long long per_try = 2ull * (unsigned)D + 1ull;
+    Rng rng{key, ctr0};
     float x[MRPOP_MAX_LINKS];
     const bool informed = C.mode == 1 && C.c_best < INFINITY && C.c_best > S.c_min;
     bool ok = false;
     if (informed) {
+        rng.ctr = ctr0 + (unsigned long long)tr * per_try;
         // Direct sampling of the prolate hyperspheroid (foci start and goal,
         // transverse diameter c_best): uniform in the unit ball, scaled by the
         // radii, reflected so that e1 maps to the start->goal axis, centred.
         const float r1 = 0.5f * C.c_best;
         const float r2 = 0.5f * sqrtf(fmaxf(C.c_best * C.c_best - S.c_min * S.c_min, 0.f));
-        for (int tr = 0; tr < kInformedTries && !ok; ++tr) {
-            float n2 = 0.f;
-            for (int d = 0; d < D; ++d) {
-                x[d] = rng.normal();
-                n2 = fmaf(x[d], x[d], n2);
-            }
-            const float rad = powf(rng.uniform(), 1.0f / (float)D) / sqrtf(fmaxf(n2, 1e-30f));
-            for (int d = 0; d < D; ++d) x[d] *= rad * (d == 0 ? r1 : r2);
-            // Householder reflection with w = e1 - axis
-            float ww = 0.f, wx = 0.f;
-            for (int d = 0; d < D; ++d) {
-                const float w = (d == 0 ? 1.f : 0.f) - S.axis[d];
-                ww = fmaf(w, w, ww);
-                wx = fmaf(w, x[d], wx);
-            }
-            const float f = ww > 1e-12f ? 2.f * wx / ww : 0.f;
-            ok = true;
-            for (int d = 0; d < D; ++d) {
-                const float w = (d == 0 ? 1.f : 0.f) - S.axis[d];
-                x[d] = S.centre[d] + x[d] - f * w;
-                ok = ok && x[d] >= S.q_lo[d] && x[d] <= S.q_hi[d];
-            }
+        float n2 = 0.f;
+        for (int d = 0; d < D; ++d) {
+            x[d] = rng.normal();
+            n2 = fmaf(x[d], x[d], n2);
+        }
+        const float rad = powf(rng.uniform(), 1.0f / (float)D) / sqrtf(fmaxf(n2, 1e-30f));
+        for (int d = 0; d < D; ++d) x[d] *= rad * (d == 0 ? r1 : r2);
+        // Householder reflection with w = e1 - axis
+        float ww = 0.f, wx = 0.f;
+        for (int d = 0; d < D; ++d) {
+            const float w = (d == 0 ? 1.f : 0.f) - S.axis[d];
+            ww = fmaf(w, w, ww);
+            wx = fmaf(w, x[d], wx);
+        }
+        const float f = ww > 1e-12f ? 2.f * wx / ww : 0.f;
+        ok = true;
+        for (int d = 0; d < D; ++d) {
+            const float w = (d == 0 ? 1.f : 0.f) - S.axis[d];
+            x[d] = S.centre[d] + x[d] - f * w;
+            ok = ok && x[d] >= S.q_lo[d] && x[d] <= S.q_hi[d];
         }
     }
+    // the first accepted try, or the last lane after all were rejected
+    const unsigned acc = __ballot_sync(half, ok) & half;
+    const int first = acc ? (__ffs(acc) - 1) & 15 : kInformedTries - 1;
+    if (tr != first) return;
+    if (!informed) rng.ctr = ctr0;
     if (!ok)
         for (int d = 0; d < D; ++d) x[d] = S.q_lo[d] + rng.uniform() * (S.q_hi[d] - S.q_lo[d]);
     for (int d = 0; d < D; ++d) S.qrand[(size_t)d * B + i] = x[d];
@@ -169,8 +183,9 @@ __device__ __forceinline__ void sample_body(const Slot &S, int i) {
     }
 }
 
+// 16 samples per block of 256 threads
 __global__ void k_sample(const Slot *__restrict__ slots) {
-    sample_body(slots[blockIdx.y], blockIdx.x * blockDim.x + threadIdx.x);
+    sample_body(slots[blockIdx.y], (blockIdx.x * blockDim.x + threadIdx.x) / kInformedTries);
 }
 
 // NEAREST over one of the slot's trees (pass 0: expanded tree with q_rand and
@@ -444,17 +459,27 @@ __global__ void k_solution(const Slot *__restrict__ slots) {
 // One thread follows the parents; the configurations are written to
 // out_q [cap][D] in that order (reversed to start -> goal by the host when the
 // expanded tree was the goal tree).
+// One thread follows the parents; the block then copies the configurations.
 __device__ __forceinline__ void extract_body(const Slot &S, int it, int *scratch, float *out_q,
                                              int cap, int *len_out) {
+    __shared__ int s_na, s_n;
     const int a = S.ctrl->tree_a, b = 1 - a, D = S.D;
-    int na = 0;
-    for (int v = S.newidx[it]; v >= 0 && na < cap; v = S.tpar[a][v]) scratch[na++] = v;
-    int n = 0;
-    for (int k = na - 1; k >= 0; --k, ++n)
-        for (int d = 0; d < D; ++d) out_q[(size_t)n * D + d] = S.tq[a][(size_t)d * S.tcap + scratch[k]];
-    for (int v = (int)S.conn[it]; v >= 0 && n < cap; v = S.tpar[b][v], ++n)
-        for (int d = 0; d < D; ++d) out_q[(size_t)n * D + d] = S.tq[b][(size_t)d * S.tcap + v];
-    *len_out = n;
+    if (threadIdx.x == 0) {
+        int n = 0;
+        for (int v = S.newidx[it]; v >= 0 && n < cap; v = S.tpar[a][v]) scratch[n++] = v;
+        s_na = n;
+        for (int v = (int)S.conn[it]; v >= 0 && n < cap; v = S.tpar[b][v]) scratch[n++] = v;
+        s_n = n;
+        *len_out = n;
+    }
+    __syncthreads();
+    const int na = s_na, n = s_n;
+    for (int i = threadIdx.x; i < n * D; i += blockDim.x) {
+        const int k = i / D, d = i - k * D;
+        const bool first = k < na;  // root_a .. z_new, the walk reversed
+        const int t = first ? a : b, v = scratch[first ? na - 1 - k : k];
+        out_q[i] = S.tq[t][(size_t)d * S.tcap + v];
+    }
 }
 
 __global__ void k_extract(const Slot *__restrict__ slots, int it, int *scratch, float *out_q,
@@ -1329,7 +1354,7 @@ static mrpop_status try_incumbent(Planner *pl, const Slot *d_slot, int it, int t
                                   cudaStream_t st, double t_now, bool *accepted) {
     *accepted = false;
     const int cap = 2 * pl->tcap + 2, D = pl->D;
-    k_extract<<<1, 1, 0, st>>>(d_slot, it, pl->d_path, pl->d_pathq, cap, pl->d_len);
+    k_extract<<<1, 128, 0, st>>>(d_slot, it, pl->d_path, pl->d_pathq, cap, pl->d_len);
     PL_TRY(cudaGetLastError());
     int len = 0;
     PL_TRY(cudaMemcpyAsync(&len, pl->d_len, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1474,7 +1499,7 @@ static mrpop_status batch_config(Batch &bt) {
 static mrpop_status enqueue_step(Batch &bt, cudaStream_t st) {
     const int n = bt.n;
     const dim3 g1((kStepIters + 127) / 128, n), gq(kStepIters / kPQB, n);
-    k_sample<<<g1, 128, 0, st>>>(bt.d_slots);
+    k_sample<<<dim3(kStepIters * kInformedTries / 256, n), 256, 0, st>>>(bt.d_slots);
     k_nearest<0><<<gq, kPThreads, 0, st>>>(bt.d_slots);
     k_oracle<<<g1, 128, 0, st>>>(bt.d_slots);
     PL_TRY(cudaGetLastError());
@@ -1770,6 +1795,7 @@ struct PState {
     double c_best, target;
     unsigned long long seed;
     int n_per_round, rcap;
+    int step_edges;            // edges per validation chunk of a search step
     float res4;                // resolution / 4 (fine re-check)
     // incumbent candidate of the current step
     int cand_len, fine_M, fine_done, fine_cnt, fine_bad, accepted;
@@ -1816,11 +1842,20 @@ __device__ __forceinline__ unsigned long long gtimer() {
 
 __device__ __forceinline__ int chunks_of(int n, int per) { return n <= 0 ? 0 : (n + per - 1) / per; }
 
-// Validation of edges [chunk * per, chunk * per + per) of vp (count edges in all).
+// Validation of edges [chunk * per, chunk * per + per) of vp (count edges in
+// all).  With two warps or more per edge an edge's tiles are shared among them.
+// s_next: kPerWarps ints of shared memory.
 __device__ __noinline__ void val_chunk(const VParams &vp, int chunk, int per, int count,
                                        float4 *sm4, int *s_next) {
-    if (threadIdx.x == 0) *s_next = 0;
+    const int tid = threadIdx.x;
+    if (tid < kPerWarps) s_next[tid] = 0;  // (visible after the tables' barrier)
     const int e0 = chunk * per, e1 = min(count, e0 + per);
+    if (2 * (e1 - e0) <= vp.warps) {
+        vb::verdict_body<true, true>(vp, sm4, e0, e1, s_next);
+        __syncthreads();
+        if (tid < e1 - e0) vp.valid[e0 + tid] = s_next[tid] == 0;
+        return;
+    }
     vb::verdict_body<true>(vp, sm4, e0, e1, s_next);
     __syncthreads();
 }
@@ -1856,9 +1891,7 @@ __device__ void solution_candidate(PState &ps, double *red) {
     const unsigned long long key = S.ctrl->best_key;
     if (tid == 0) ps.fine_M = 0;
     if (key == ~0ull) return;
-    if (tid == 0)
-        extract_body(S, (int)(key & 0xffffffffu), ps.scratch, ps.cand_path, ps.path_cap,
-                     &ps.cand_len);
+    extract_body(S, (int)(key & 0xffffffffu), ps.scratch, ps.cand_path, ps.path_cap, &ps.cand_len);
     __syncthreads();
     const int len = ps.cand_len, D = ps.D;
     if (S.ctrl->tree_a == 1)  // the expanded tree was the goal tree: reverse
@@ -2001,19 +2034,19 @@ __device__ void run_chunk(PState &ps, int kind, int c, float4 *sm4, NnShared<kPe
             link_body(ps.jobs[r], *reinterpret_cast<LinkShared *>(sm4));
             break;
         }
-        case PK_ST_SAMPLE: sample_body(S, tid); break;
+        case PK_ST_SAMPLE: sample_body(S, (c * kPerThreads + tid) / kInformedTries); break;
         case PK_ST_NN0: nearest_body<0, kPerThreads>(S, c, nn); break;
         case PK_ST_ORACLE: oracle_body(S, tid); break;
-        case PK_ST_VAL1: val_chunk(ps.vp[0], c, kPerEdges, kStepIters, sm4, s_next); break;
+        case PK_ST_VAL1: val_chunk(ps.vp[0], c, ps.step_edges, kStepIters, sm4, s_next); break;
         case PK_ST_INSERT: insert_body(S, wsum); break;
         case PK_ST_NN1: nearest_body<1, kPerThreads>(S, c, nn); break;
         case PK_ST_CONN: conn_prep_body(S, tid); break;
-        case PK_ST_VAL2: val_chunk(ps.vp[1], c, kPerEdges, kStepIters, sm4, s_next); break;
+        case PK_ST_VAL2: val_chunk(ps.vp[1], c, ps.step_edges, kStepIters, sm4, s_next); break;
         case PK_ST_SOLUTION:
             solution_body(S, tid);
             solution_candidate(ps, red);
             break;
-        case PK_FINE_VAL: val_chunk(ps.vp[2], c, kPerEdges, ps.fine_cnt, sm4, s_next); break;
+        case PK_FINE_VAL: val_chunk(ps.vp[2], c, ps.step_edges, ps.fine_cnt, sm4, s_next); break;
         case PK_FINE_ACCEPT: fine_accept(ps); break;
         default: break;
     }
@@ -2053,7 +2086,7 @@ __device__ unsigned long long start_step(PState &ps) {
     C.best_key = ~0ull;
     C.overflow = 0;
     if (C.mode == 2) return 0ull;  // an idle step changes nothing: the outer iteration ends
-    return phase_word(PK_ST_SAMPLE, 1);
+    return phase_word(PK_ST_SAMPLE, kStepIters * kInformedTries / kPerThreads);
 }
 
 __device__ PDecision begin_outer(PState &ps, unsigned long long now, unsigned long long deadline);
@@ -2160,19 +2193,19 @@ __device__ PDecision decide(PState &ps, int kind, unsigned long long now,
         }
         case PK_ST_SAMPLE: return {phase_word(PK_ST_NN0, kStepIters / kPQB), 0};
         case PK_ST_NN0: return {phase_word(PK_ST_ORACLE, 1), 0};
-        case PK_ST_ORACLE: return {phase_word(PK_ST_VAL1, kStepIters / kPerEdges), 0};
+        case PK_ST_ORACLE: return {phase_word(PK_ST_VAL1, kStepIters / ps.step_edges), 0};
         case PK_ST_VAL1: return {phase_word(PK_ST_INSERT, 1), 0};
         case PK_ST_INSERT: return {phase_word(PK_ST_NN1, kStepIters / kPQB), 0};
         case PK_ST_NN1: return {phase_word(PK_ST_CONN, 1), 0};
-        case PK_ST_CONN: return {phase_word(PK_ST_VAL2, kStepIters / kPerEdges), 0};
+        case PK_ST_CONN: return {phase_word(PK_ST_VAL2, kStepIters / ps.step_edges), 0};
         case PK_ST_VAL2: return {phase_word(PK_ST_SOLUTION, 1), 0};
         case PK_ST_SOLUTION:
-            if (ps.fine_M > 0) return {phase_word(PK_FINE_VAL, chunks_of(ps.fine_cnt, kPerEdges)), 0};
+            if (ps.fine_M > 0) return {phase_word(PK_FINE_VAL, chunks_of(ps.fine_cnt, ps.step_edges)), 0};
             return after_step(ps, false, now, deadline);
         case PK_FINE_VAL: return {phase_word(PK_FINE_ACCEPT, 1), 0};
         case PK_FINE_ACCEPT:
             if (ps.fine_bad) return after_step(ps, false, now, deadline);
-            if (!ps.accepted) return {phase_word(PK_FINE_VAL, chunks_of(ps.fine_cnt, kPerEdges)), 0};
+            if (!ps.accepted) return {phase_word(PK_FINE_VAL, chunks_of(ps.fine_cnt, ps.step_edges)), 0};
             return after_step(ps, true, now, deadline);
         default: return {phase_word(PK_DONE, 0), 0};
     }
@@ -2183,7 +2216,8 @@ __global__ void __launch_bounds__(kPerThreads) k_persistent(const PLaunch L) {
     __shared__ NnShared<kPerThreads> nn;
     __shared__ int wsum[kPerWarps];
     __shared__ double red[kPerThreads];
-    __shared__ int s_q, s_kind, s_chunk, s_total, s_last, s_exit, s_next, s_reset;
+    __shared__ int s_q, s_kind, s_chunk, s_total, s_last, s_exit, s_reset;
+    __shared__ int s_next[kPerWarps];
     __shared__ unsigned long long s_t0, s_word;
     const int tid = threadIdx.x;
     if (tid == 0) {
@@ -2236,7 +2270,7 @@ __global__ void __launch_bounds__(kPerThreads) k_persistent(const PLaunch L) {
         __threadfence();  // acquire: the phase's inputs, written by other CTAs
         PState &ps = L.states[s_q];
         const unsigned long long tc0 = tid == 0 ? gtimer() : 0ull;
-        run_chunk(ps, s_kind, s_chunk, per_sm4, nn, wsum, &s_next, red);
+        run_chunk(ps, s_kind, s_chunk, per_sm4, nn, wsum, s_next, red);
         __threadfence();  // release: this chunk's results
         __syncthreads();
         if (tid == 0) {
@@ -2425,6 +2459,12 @@ static mrpop_status plan_batch_persistent(mrpop_problem *const *ps, int n, doubl
     if (bps < 1) return set_error(MRPOP_EINVAL, "plan_batch: persistent kernel does not fit an SM");
     const int ctas = g_per_ctas.load() > 0 ? g_per_ctas.load() : sms * bps;
 
+    // edges per validation chunk of a search step: 32 when the problems alone
+    // fill the CTAs, fewer while their chunks would not (twelve problems of 2-8
+    // arms on 304 CTAs: 8 edges, 112 us a chunk instead of 352); the verdicts do not depend on it
+    int step_edges = kPerEdges;
+    while (step_edges > 1 && (int64_t)n * (kStepIters / step_edges) <= ctas) step_edges /= 2;
+
     // per-problem state from the host mirrors (each call starts with a
     // roadmap round, as Alg. 1 does)
     std::vector<PState> hs(n);
@@ -2465,6 +2505,7 @@ static mrpop_status plan_batch_persistent(mrpop_problem *const *ps, int n, doubl
         s.seed = pl->seed;
         s.n_per_round = pl->n_per_round;
         s.rcap = pl->rcap;
+        s.step_edges = step_edges;
         s.res4 = 0.25f * pl->p->cfg.resolution;
         s.slot = b.slot;
         s.jobs = b.jobs;

@@ -924,7 +924,9 @@ __device__ __forceinline__ bool link_obstacles(const float4 *tab, const Tables &
 // GROUP: the block's warps share one edge (edge blockIdx.x), tile after tile in
 // turn, for batches of so few edges that an edge per warp would leave most of
 // the chip idle: the time is then that of the longest edge, one tile after
-// another.  The caller gives a shared flag (zero) in s_next.
+// another.  The caller gives a shared flag (zero) in s_next.  With LOCAL too, the
+// warps of each of the edges [e0, e1) are (P.warps / their number) in a row, s_next
+// holds a zero flag for each, and the caller turns the flags into verdicts.
 template <bool LOCAL, bool GROUP = false>
 __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int e0 = 0, int e1 = 0,
                                              int *s_next = nullptr) {
@@ -950,9 +952,13 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
     const float m = P.margin;
     if (lane == 0) ad[D] = make_float2(0.f, 0.f);
     const bool pairs = K > 1 || t.selfcol;
+    const int split = GROUP ? (LOCAL ? P.warps / max(e1 - e0, 1) : P.warps) : 1;  // warps per edge
     for (;;) {
         int e = 0;
-        if (GROUP) {
+        if (GROUP && LOCAL) {
+            e = e0 + warp / split;
+            if (e >= e1) return;
+        } else if (GROUP) {
             e = blockIdx.x;
         } else {
             if (lane == 0) e = LOCAL ? e0 + atomicAdd(s_next, 1) : atomicAdd(&P.work[0], 1);
@@ -976,8 +982,9 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
         const int T = too_long ? 0 : (n >> 5) + 1;  // ceil((n + 1) / 32)
         bool edge_hit = too_long;
 
-        for (int tile = GROUP ? warp : 0; tile < T && !edge_hit; tile += GROUP ? P.warps : 1) {
-            if (GROUP && *(volatile int *)s_next) break;  // another warp's tile collides
+        volatile int *flag = GROUP ? s_next + (LOCAL ? e - e0 : 0) : nullptr;
+        for (int tile = GROUP ? warp % split : 0; tile < T && !edge_hit; tile += split) {
+            if (GROUP && *flag) break;  // another warp's tile collides
             int k = P.order ? tile * 32 + lane : tile + T * lane;
             k = min(k, n);
             // (k = 0 apart: a zero numerator sends the whole warp through the
@@ -1117,9 +1124,10 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
             }
         }
         if (GROUP) {
-            if (lane == 0 && edge_hit) *(volatile int *)s_next = 1;
+            if (lane == 0 && edge_hit) *flag = 1;
+            if (LOCAL) return;
             __syncthreads();
-            edge_hit = *(volatile int *)s_next != 0;
+            edge_hit = *flag != 0;
         }
         if (lane == 0 && (!GROUP || warp == 0)) {
             P.valid[e] = edge_hit ? 0 : 1;

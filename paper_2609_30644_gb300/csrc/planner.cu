@@ -1916,16 +1916,30 @@ __device__ void solution_candidate(PState &ps, double *red) {
     }
     red[tid] = c;
     __syncthreads();
+    bool better = false;
     if (tid == 0) {
         double cost = 0.0;
-        for (int k = 0; k < blockDim.x; ++k) cost += red[k];
+#pragma unroll 16
+        for (int k = 0; k < kPerThreads; ++k) cost += red[k];
         ps.cand_cost = cost;
-        if (cost < ps.c_best && len >= 2) {
-            int M = 0;
-            for (int j = 0; j + 1 < len; ++j) {
-                ps.scratch[j] = M;  // the path indices are no longer needed
-                M += ps.seg_parts[j];
+        better = cost < ps.c_best && len >= 2;
+    }
+    // the segments' offsets, 32 at a time (the path indices in scratch are no
+    // longer needed)
+    if (tid < 32 && __shfl_sync(0xffffffffu, better ? 1 : 0, 0)) {
+        int M = 0;
+        for (int j0 = 0; j0 + 1 < len; j0 += 32) {
+            const int j = j0 + tid, own = j + 1 < len ? ps.seg_parts[j] : 0;
+            int x = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (tid >= o) x += y;
             }
+            if (j + 1 < len) ps.scratch[j] = M + x - own;
+            M += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (tid == 0) {
             ps.fine_M = M;
             ps.fine_done = 0;
             ps.fine_bad = 0;
@@ -2029,7 +2043,16 @@ __device__ void run_chunk(PState &ps, int kind, int c, float4 *sm4, NnShared<kPe
         }
         case PK_RM_NB: rmb_neighbors_body(ps.jobs[r], c * kPerWarps + (tid >> 5)); break;
         case PK_RM_EDGES: rmb_edges_body(ps.jobs[r], c * kPerThreads + tid); break;
-        case PK_RM_VALE: val_chunk(ps.vp[3 + ps.K + r], c, kPerEdges, ps.jobs[r].emax, sm4, s_next); break;
+        case PK_RM_VALE: {
+            // (most slots of a young roadmap's neighbour lists are unused: a
+            // chunk without an edge needs no tables and no verdicts, which are
+            // read for edges only)
+            const RmJob &J = ps.jobs[r];
+            const int e = c * kPerEdges + tid;
+            if (!__syncthreads_or(tid < kPerEdges && e < J.emax && J.ea[e] >= 0)) break;
+            val_chunk(ps.vp[3 + ps.K + r], c, kPerEdges, J.emax, sm4, s_next);
+            break;
+        }
         case PK_RM_LINK: {
             link_body(ps.jobs[r], *reinterpret_cast<LinkShared *>(sm4));
             break;

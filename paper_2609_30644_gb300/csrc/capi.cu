@@ -496,9 +496,17 @@ mrpop_status mrpop::create_problem(const mrpop_robot *robots, int32_t K,
     p->num_sms = v;
     cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
     p->smem_optin = (size_t)v;
-    if ((e = cudaMalloc(&p->dev.blob, p->h_blob.size() * sizeof(float))) != cudaSuccess)
+    // one allocation and one copy: tables, joint limits, work counter (zero)
+    std::vector<float> dev_tables = p->h_blob;
+    dev_tables.insert(dev_tables.end(), p->q_lo.begin(), p->q_lo.end());
+    dev_tables.insert(dev_tables.end(), p->q_hi.begin(), p->q_hi.end());
+    dev_tables.resize(dev_tables.size() + 4, 0.f);
+    if ((e = cudaMalloc(&p->dev.blob, dev_tables.size() * sizeof(float))) != cudaSuccess)
         return fail(cuda_error(e, "cudaMalloc(tables)"));
-    if ((e = cudaMemcpy(p->dev.blob, p->h_blob.data(), p->h_blob.size() * sizeof(float),
+    p->dev.q_lo = reinterpret_cast<float *>(p->dev.blob + t.n_f4);
+    p->dev.q_hi = p->dev.q_lo + L;
+    p->dev.edge_counter = reinterpret_cast<int *>(p->dev.q_hi + L);
+    if ((e = cudaMemcpy(p->dev.blob, dev_tables.data(), dev_tables.size() * sizeof(float),
                         cudaMemcpyHostToDevice)) != cudaSuccess)
         return fail(cuda_error(e, "cudaMemcpy(tables)"));
     if (build) {
@@ -510,19 +518,9 @@ mrpop_status mrpop::create_problem(const mrpop_robot *robots, int32_t K,
             launch_field(p->dev.t, p->dev.blob, edge, shrink, (float)unit, p->dev.field, nullptr);
         if (s != MRPOP_OK) return fail(s);
     }
-    if ((e = cudaMalloc(&p->dev.q_lo, sizeof(float) * L)) != cudaSuccess ||
-        (e = cudaMalloc(&p->dev.q_hi, sizeof(float) * L)) != cudaSuccess)
-        return fail(cuda_error(e, "cudaMalloc(limits)"));
-    cudaMemcpy(p->dev.q_lo, p->q_lo.data(), sizeof(float) * L, cudaMemcpyHostToDevice);
-    if ((e = cudaMemcpy(p->dev.q_hi, p->q_hi.data(), sizeof(float) * L,
-                        cudaMemcpyHostToDevice)) != cudaSuccess)
-        return fail(cuda_error(e, "cudaMemcpy(limits)"));
-    if ((e = cudaMalloc(&p->dev.edge_counter, sizeof(int) * 4)) != cudaSuccess)
-        return fail(cuda_error(e, "cudaMalloc(counter)"));
-    if ((e = cudaMemset(p->dev.edge_counter, 0, sizeof(int) * 4)) != cudaSuccess)
-        return fail(cuda_error(e, "cudaMemset(counter)"));
-    // the field and the counter are used on any stream from here on
-    if ((e = cudaStreamSynchronize(nullptr)) != cudaSuccess)
+    // the tables and the field are used on any stream from here on (the planner
+    // synchronises once for all of its sub-problems)
+    if (!share && (e = cudaStreamSynchronize(nullptr)) != cudaSuccess)
         return fail(cuda_error(e, "problem tables"));
     // a launch tuned earlier for a problem of this shape (mrpop_autotune)
     std::vector<int> tuned;
@@ -538,14 +536,11 @@ mrpop_status mrpop::create_problem(const mrpop_robot *robots, int32_t K,
 
 extern "C" mrpop_status mrpop_destroy_problem(mrpop_problem *p) {
     if (!p) return MRPOP_OK;
-    if (p->dev.blob || p->dev.edge_counter) cudaDeviceSynchronize();
+    if (p->dev.blob) cudaDeviceSynchronize();
     destroy_planner(p->planner);
     p->planner = nullptr;
     cudaFree(p->dev.blob);
     cudaFree(p->dev.field);
-    cudaFree(p->dev.q_lo);
-    cudaFree(p->dev.q_hi);
-    cudaFree(p->dev.edge_counter);
     delete p;
     return MRPOP_OK;
 }

@@ -855,9 +855,55 @@ __global__ void k_tree_reset(const Slot *__restrict__ slots) { tree_reset_body(s
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-template <class T>
-static cudaError_t dalloc(T **p, size_t n) {
-    return cudaMalloc((void **)p, sizeof(T) * std::max<size_t>(n, 1));
+// Device buffers of one owner in one allocation: request() notes them,
+// commit() allocates the sum and sets the pointers.  A planner's 30 to 150
+// buffers were as many allocations and frees, of which those of 2 MB and more
+// map and unmap memory: twelve planning requests of 2-8 arms spent 28 ms on the
+// host beside an 18 ms kernel, and 10 ms now.
+struct DeviceArena {
+    struct Want {
+        void **p;
+        size_t bytes;
+    };
+    std::vector<Want> wants;
+    char *base = nullptr;
+    size_t bytes = 0;
+    template <class T>
+    void request(T **p, size_t n) {
+        wants.push_back({(void **)p, sizeof(T) * std::max<size_t>(n, 1)});
+    }
+    // zero: clear the whole allocation (on the legacy stream)
+    cudaError_t commit(bool zero) {
+        bytes = 0;
+        for (const Want &w : wants) bytes += (w.bytes + 255) & ~(size_t)255;
+        cudaError_t e = cudaMalloc((void **)&base, std::max<size_t>(bytes, 256));
+        if (e != cudaSuccess) {
+            base = nullptr;
+            wants.clear();
+            return e;
+        }
+        size_t at = 0;
+        for (const Want &w : wants) {
+            *w.p = base + at;
+            at += (w.bytes + 255) & ~(size_t)255;
+        }
+        wants.clear();
+        return zero ? cudaMemsetAsync(base, 0, bytes, nullptr) : cudaSuccess;
+    }
+    void release() {
+        cudaFree(base);
+        base = nullptr;
+        bytes = 0;
+    }
+};
+
+// The robots' start and goal (roadmap vertices 0 and 1).
+__global__ void k_roadmap_roots(const Slot S) {
+    const int k = blockIdx.x;
+    for (int d = threadIdx.x; d < S.dof[k]; d += blockDim.x) {
+        S.rm_q[k][(size_t)d * S.rcap] = S.start[S.qoff[k] + d];
+        S.rm_q[k][(size_t)d * S.rcap + 1] = S.goal[S.qoff[k] + d];
+    }
 }
 
 struct RobotRoadmap {
@@ -880,6 +926,7 @@ struct RobotRoadmap {
 
 // Device buffers of the persistent form, per planner (allocated on first use).
 struct PerBuffers {
+    DeviceArena arena;
     Slot *slot = nullptr;
     RmJob *jobs = nullptr;
     VParams *vp = nullptr;
@@ -897,13 +944,12 @@ struct PerBuffers {
 };
 
 static void per_free(PerBuffers &b) {
-    cudaFree(b.slot); cudaFree(b.jobs); cudaFree(b.vp); cudaFree(b.seg_parts); cudaFree(b.best);
-    cudaFree(b.trace_c); cudaFree(b.trace_ns); cudaFree(b.trace_it); cudaFree(b.hist);
-    cudaFree(b.hist_len);
+    b.arena.release();
     b = PerBuffers{};
 }
 
 struct Planner {
+    DeviceArena arena;        // every buffer below but the fine re-check's
     mrpop_problem *p = nullptr;
     mrpop_problem *fine = nullptr;  // same scene at resolution / 4
     int K = 0, D = 0, rcap = 0, tcap = 0, n_per_round = 0;
@@ -993,24 +1039,9 @@ void destroy_planner(Planner *pl) {
 
 // Frees every device buffer of the planner; host-side results stay.
 static void free_device(Planner *pl) {
-    for (auto &r : pl->rm) {
-        mrpop_destroy_problem(r.sub);
-        cudaFree(r.q); cudaFree(r.adj); cudaFree(r.deg); cudaFree(r.cand); cudaFree(r.gq);
-        cudaFree(r.ea_q); cudaFree(r.eb_q); cudaFree(r.cvalid); cudaFree(r.evalid);
-        cudaFree(r.nb); cudaFree(r.cnt); cudaFree(r.ea); cudaFree(r.eb);
-        cudaFree(r.level); cudaFree(r.d_conn);
-    }
+    for (auto &r : pl->rm) mrpop_destroy_problem(r.sub);
     mrpop_destroy_problem(pl->fine);
-    cudaFree(pl->rm_n);
-    for (int t = 0; t < 2; ++t) {
-        cudaFree(pl->tq[t]); cudaFree(pl->tpar[t]); cudaFree(pl->trmv[t]);
-    }
-    cudaFree(pl->tn); cudaFree(pl->buf); cudaFree(pl->near); cudaFree(pl->conn);
-    cudaFree(pl->rmvnew); cudaFree(pl->newidx); cudaFree(pl->valid1); cudaFree(pl->valid2);
-    cudaFree(pl->d_lo); cudaFree(pl->d_hi); cudaFree(pl->d_start); cudaFree(pl->d_goal);
-    cudaFree(pl->d_centre); cudaFree(pl->d_axis); cudaFree(pl->ctrl); cudaFree(pl->d_path);
-    cudaFree(pl->d_pathq);
-    cudaFree(pl->d_len);
+    pl->arena.release();
     cudaFree(pl->fine_qa);
     cudaFree(pl->fine_qb);
     cudaFree(pl->fine_v);
@@ -1091,68 +1122,46 @@ static mrpop_status planner_init(mrpop_problem *p, Planner **out) {
         ST_TRY(make_sub(p, k, p->cfg.resolution, &r.sub));
         const int nc = kOversample * pl->n_per_round;
         const int E = pl->n_per_round * kKmax;
-        PL_TRY(dalloc(&r.q, (size_t)dof * rcap));
-        PL_TRY(dalloc(&r.adj, (size_t)rcap * kKmax));
-        PL_TRY(dalloc(&r.deg, (size_t)rcap));
-        PL_TRY(cudaMemset(r.deg, 0, sizeof(int) * rcap));
-        PL_TRY(dalloc(&r.cand, (size_t)dof * nc));
-        PL_TRY(dalloc(&r.cvalid, (size_t)nc));
-        PL_TRY(dalloc(&r.gq, (size_t)dof * pl->n_per_round + 2 * dof));
-        PL_TRY(dalloc(&r.nb, (size_t)(pl->n_per_round + 2) * kKmax));
-        PL_TRY(dalloc(&r.cnt, (size_t)pl->n_per_round + 2));
-        PL_TRY(dalloc(&r.ea_q, (size_t)dof * (E + 2 * kKmax)));
-        PL_TRY(dalloc(&r.eb_q, (size_t)dof * (E + 2 * kKmax)));
-        PL_TRY(dalloc(&r.evalid, (size_t)E + 2 * kKmax));
-        PL_TRY(dalloc(&r.ea, (size_t)E + 2 * kKmax));
-        PL_TRY(dalloc(&r.eb, (size_t)E + 2 * kKmax));
-        PL_TRY(dalloc(&r.level, (size_t)rcap));
-        PL_TRY(dalloc(&r.d_conn, 1));
-        PL_TRY(cudaMemset(r.d_conn, 0, sizeof(int)));
-        // vertices 0 and 1: the robot's start and goal
-        for (int d = 0; d < dof; ++d) {
-            PL_TRY(cudaMemcpy(r.q + (size_t)d * rcap, &p->start[qoff + d], sizeof(float),
-                              cudaMemcpyHostToDevice));
-            PL_TRY(cudaMemcpy(r.q + (size_t)d * rcap + 1, &p->goal[qoff + d], sizeof(float),
-                              cudaMemcpyHostToDevice));
-        }
+        pl->arena.request(&r.q, (size_t)dof * rcap);
+        pl->arena.request(&r.adj, (size_t)rcap * kKmax);
+        pl->arena.request(&r.deg, (size_t)rcap);
+        pl->arena.request(&r.cand, (size_t)dof * nc);
+        pl->arena.request(&r.cvalid, (size_t)nc);
+        pl->arena.request(&r.gq, (size_t)dof * pl->n_per_round + 2 * dof);
+        pl->arena.request(&r.nb, (size_t)(pl->n_per_round + 2) * kKmax);
+        pl->arena.request(&r.cnt, (size_t)pl->n_per_round + 2);
+        pl->arena.request(&r.ea_q, (size_t)dof * (E + 2 * kKmax));
+        pl->arena.request(&r.eb_q, (size_t)dof * (E + 2 * kKmax));
+        pl->arena.request(&r.evalid, (size_t)E + 2 * kKmax);
+        pl->arena.request(&r.ea, (size_t)E + 2 * kKmax);
+        pl->arena.request(&r.eb, (size_t)E + 2 * kKmax);
+        pl->arena.request(&r.level, (size_t)rcap);
+        pl->arena.request(&r.d_conn, 1);
         r.n = 2;
-        ST_TRY(make_vparams(r.sub, r.cand, r.cand, nc, r.cvalid, &r.vp_c, &r.vs_c, &r.vw_c));
-        ST_TRY(make_vparams(r.sub, r.ea_q, r.eb_q, E + 2 * kKmax, r.evalid, &r.vp_e, &r.vs_e,
-                            &r.vw_e));
         pl->slot.dof[k] = dof;
         pl->slot.qoff[k] = qoff;
-        pl->slot.rm_q[k] = r.q;
-        pl->slot.rm_adj[k] = r.adj;
-        pl->slot.rm_deg[k] = r.deg;
         qoff += dof;
     }
-    PL_TRY(dalloc(&pl->rm_n, K));
-    std::vector<int> twos(K, 2);
-    PL_TRY(cudaMemcpy(pl->rm_n, twos.data(), sizeof(int) * K, cudaMemcpyHostToDevice));
     for (int t = 0; t < 2; ++t) {
-        PL_TRY(dalloc(&pl->tq[t], (size_t)(D + 1) * tcap));
-        PL_TRY(dalloc(&pl->tpar[t], (size_t)tcap));
-        PL_TRY(dalloc(&pl->trmv[t], (size_t)K * tcap));
+        pl->arena.request(&pl->tq[t], (size_t)(D + 1) * tcap);
+        pl->arena.request(&pl->tpar[t], (size_t)tcap);
+        pl->arena.request(&pl->trmv[t], (size_t)K * tcap);
     }
-    PL_TRY(dalloc(&pl->tn, 2));
+    pl->arena.request(&pl->tn, 2);
     // step buffers: qrand, qnear, qnew, qconn [D][B]; crand, gnew, budget2 [B]
-    PL_TRY(dalloc(&pl->buf, (size_t)4 * D * B + 3 * B));
-    PL_TRY(dalloc(&pl->near, B));
-    PL_TRY(dalloc(&pl->conn, B));
-    PL_TRY(dalloc(&pl->rmvnew, (size_t)K * B));
-    PL_TRY(dalloc(&pl->newidx, B));
-    PL_TRY(dalloc(&pl->valid1, B));
-    PL_TRY(dalloc(&pl->valid2, B));
-    PL_TRY(dalloc(&pl->d_lo, D));
-    PL_TRY(dalloc(&pl->d_hi, D));
-    PL_TRY(dalloc(&pl->d_start, D));
-    PL_TRY(dalloc(&pl->d_goal, D));
-    PL_TRY(dalloc(&pl->d_centre, D));
-    PL_TRY(dalloc(&pl->d_axis, D));
-    PL_TRY(dalloc(&pl->ctrl, 1));
-    PL_TRY(dalloc(&pl->d_path, (size_t)2 * tcap + 2));
-    PL_TRY(dalloc(&pl->d_pathq, (size_t)(2 * tcap + 2) * D));
-    PL_TRY(dalloc(&pl->d_len, 1));
+    pl->arena.request(&pl->buf, (size_t)4 * D * B + 3 * B);
+    pl->arena.request(&pl->near, B);
+    pl->arena.request(&pl->conn, B);
+    pl->arena.request(&pl->rmvnew, (size_t)K * B);
+    pl->arena.request(&pl->newidx, B);
+    pl->arena.request(&pl->valid1, B);
+    pl->arena.request(&pl->valid2, B);
+    float *tables = nullptr;  // limits, start, goal, centre, axis [D] each, then rm_n [K]
+    pl->arena.request(&tables, (size_t)6 * D + K);
+    pl->arena.request(&pl->ctrl, 1);
+    pl->arena.request(&pl->d_path, (size_t)2 * tcap + 2);
+    pl->arena.request(&pl->d_pathq, (size_t)(2 * tcap + 2) * D);
+    pl->arena.request(&pl->d_len, 1);
     std::vector<float> centre(D), axis(D);
     double cmin2 = 0.0;
     for (int d = 0; d < D; ++d) {
@@ -1163,12 +1172,36 @@ static mrpop_status planner_init(mrpop_problem *p, Planner **out) {
     const double cmin = std::sqrt(cmin2);
     for (int d = 0; d < D; ++d)
         axis[d] = cmin > 0 ? (float)(((double)p->goal[d] - p->start[d]) / cmin) : (d == 0 ? 1.f : 0.f);
-    PL_TRY(cudaMemcpy(pl->d_lo, p->q_lo.data(), sizeof(float) * D, cudaMemcpyHostToDevice));
-    PL_TRY(cudaMemcpy(pl->d_hi, p->q_hi.data(), sizeof(float) * D, cudaMemcpyHostToDevice));
-    PL_TRY(cudaMemcpy(pl->d_start, p->start.data(), sizeof(float) * D, cudaMemcpyHostToDevice));
-    PL_TRY(cudaMemcpy(pl->d_goal, p->goal.data(), sizeof(float) * D, cudaMemcpyHostToDevice));
-    PL_TRY(cudaMemcpy(pl->d_centre, centre.data(), sizeof(float) * D, cudaMemcpyHostToDevice));
-    PL_TRY(cudaMemcpy(pl->d_axis, axis.data(), sizeof(float) * D, cudaMemcpyHostToDevice));
+    PL_TRY(pl->arena.commit(true));  // degrees and connected flags start at zero
+    pl->d_lo = tables;
+    pl->d_hi = tables + D;
+    pl->d_start = tables + 2 * D;
+    pl->d_goal = tables + 3 * D;
+    pl->d_centre = tables + 4 * D;
+    pl->d_axis = tables + 5 * D;
+    pl->rm_n = reinterpret_cast<int *>(tables + 6 * D);
+    std::vector<float> up(6 * (size_t)D + K);
+    for (int d = 0; d < D; ++d) {
+        up[d] = p->q_lo[d];
+        up[D + d] = p->q_hi[d];
+        up[2 * D + d] = p->start[d];
+        up[3 * D + d] = p->goal[d];
+        up[4 * D + d] = centre[d];
+        up[5 * D + d] = axis[d];
+    }
+    const int two = 2;
+    for (int k = 0; k < K; ++k) std::memcpy(&up[6 * (size_t)D + k], &two, sizeof(two));
+    PL_TRY(cudaMemcpy(tables, up.data(), sizeof(float) * up.size(), cudaMemcpyHostToDevice));
+    for (int k = 0; k < K; ++k) {
+        RobotRoadmap &r = pl->rm[k];
+        const int nc = kOversample * pl->n_per_round, E = pl->n_per_round * kKmax;
+        ST_TRY(make_vparams(r.sub, r.cand, r.cand, nc, r.cvalid, &r.vp_c, &r.vs_c, &r.vw_c));
+        ST_TRY(make_vparams(r.sub, r.ea_q, r.eb_q, E + 2 * kKmax, r.evalid, &r.vp_e, &r.vs_e,
+                            &r.vw_e));
+        pl->slot.rm_q[k] = r.q;
+        pl->slot.rm_adj[k] = r.adj;
+        pl->slot.rm_deg[k] = r.deg;
+    }
 
     Slot &S = pl->slot;
     S.K = K; S.D = D; S.rcap = rcap; S.tcap = tcap;
@@ -1194,6 +1227,10 @@ static mrpop_status planner_init(mrpop_problem *p, Planner **out) {
     S.valid1 = pl->valid1; S.valid2 = pl->valid2; S.ctrl = pl->ctrl;
     ST_TRY(make_vparams(p, S.qnear, S.qnew, B, S.valid1, &pl->vp[0], &pl->vsmem, &pl->vwarps));
     ST_TRY(make_vparams(p, S.qnew, S.qconn, B, S.valid2, &pl->vp[1], &pl->vsmem, &pl->vwarps));
+    k_roadmap_roots<<<K, 32, 0, nullptr>>>(S);
+    PL_TRY(cudaGetLastError());
+    // the sub-problems' tables and all of the above are used on other streams
+    PL_TRY(cudaStreamSynchronize(nullptr));
     pl->initialised = true;
     return MRPOP_OK;
 }
@@ -2379,17 +2416,18 @@ static mrpop_status per_buffers(Planner *pl, std::vector<VParams> &vps) {
     PerBuffers &b = pl->per;
     const int K = pl->K, D = pl->D, cap = 2 * pl->tcap + 2;
     if (!b.slot) {
-        PL_TRY(dalloc(&b.slot, 1));
-        PL_TRY(dalloc(&b.jobs, K));
-        PL_TRY(dalloc(&b.vp, 3 + 2 * K));
-        PL_TRY(dalloc(&b.seg_parts, cap));
-        PL_TRY(dalloc(&b.best, (size_t)cap * D));
-        PL_TRY(dalloc(&b.trace_c, kTraceCap));
-        PL_TRY(dalloc(&b.trace_ns, kTraceCap));
-        PL_TRY(dalloc(&b.trace_it, kTraceCap));
+        b.arena.request(&b.slot, 1);
+        b.arena.request(&b.jobs, K);
+        b.arena.request(&b.vp, 3 + 2 * K);
+        b.arena.request(&b.seg_parts, cap);
+        b.arena.request(&b.best, (size_t)cap * D);
+        b.arena.request(&b.trace_c, kTraceCap);
+        b.arena.request(&b.trace_ns, kTraceCap);
+        b.arena.request(&b.trace_it, kTraceCap);
         b.hist_floats = kHistCap * std::min(cap, 512) * D;
-        PL_TRY(dalloc(&b.hist, (size_t)b.hist_floats));
-        PL_TRY(dalloc(&b.hist_len, kHistCap));
+        b.arena.request(&b.hist, (size_t)b.hist_floats);
+        b.arena.request(&b.hist_len, kHistCap);
+        PL_TRY(b.arena.commit(false));
         if (pl->fine_cap < (size_t)kFineCap) {  // grow the fine re-check buffers
             cudaFree(pl->fine_qa);
             cudaFree(pl->fine_qb);

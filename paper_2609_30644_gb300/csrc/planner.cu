@@ -1901,19 +1901,23 @@ __device__ __noinline__ void val_chunk(const VParams &vp, int chunk, int per, in
 // at most 31 intervals at resolution / 4, as in the stepped form) into the
 // fine re-check buffers, positions e - w0.
 __device__ void fine_window(PState &ps, int w0, int w1) {
-    const int len = ps.cand_len, D = ps.D;
+    const int D = ps.D, lane = threadIdx.x & 31;
     const float *path = ps.cand_path;
-    for (int j = threadIdx.x; j + 1 < len; j += blockDim.x) {
-        const int off = ps.scratch[j], parts = ps.seg_parts[j];
-        for (int i = max(0, w0 - off); i < parts && off + i < w1; ++i) {
-            const int e = off + i - w0;
-            const double t0 = (double)i / parts, t1 = (double)(i + 1) / parts;
-            for (int d = 0; d < D; ++d) {
-                const double a = path[(size_t)j * D + d], b = path[(size_t)(j + 1) * D + d];
-                ps.fine_qa[(size_t)d * kFineCap + e] = i == 0 ? (float)a : (float)(a + t0 * (b - a));
-                ps.fine_qb[(size_t)d * kFineCap + e] =
-                    i + 1 == parts ? (float)b : (float)(a + t1 * (b - a));
-            }
+    // a warp per sub-edge, its lanes over the dimensions
+    for (int s = w0 + (threadIdx.x >> 5); s < w1; s += kPerWarps) {
+        int j = 0, hi = ps.cand_len - 1;  // the last segment whose offset is <= s
+        while (hi - j > 1) {
+            const int mid = (j + hi) >> 1;
+            if (ps.scratch[mid] <= s) j = mid;
+            else hi = mid;
+        }
+        const int i = s - ps.scratch[j], parts = ps.seg_parts[j], e = s - w0;
+        const double t0 = (double)i / parts, t1 = (double)(i + 1) / parts;
+        for (int d = lane; d < D; d += 32) {
+            const double a = path[(size_t)j * D + d], b = path[(size_t)(j + 1) * D + d];
+            ps.fine_qa[(size_t)d * kFineCap + e] = i == 0 ? (float)a : (float)(a + t0 * (b - a));
+            ps.fine_qb[(size_t)d * kFineCap + e] =
+                i + 1 == parts ? (float)b : (float)(a + t1 * (b - a));
         }
     }
 }

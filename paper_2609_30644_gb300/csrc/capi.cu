@@ -418,6 +418,19 @@ mrpop_status mrpop::create_problem(const mrpop_robot *robots, int32_t K,
         }
     }
 
+    // grid coordinates: 61,440 steps over the reach and 2,048 to spare on
+    // either side for the rounding of pc, coarser steps where the workspace
+    // lies so far out that the rounding would pass that
+    {
+        double extent = 1e-30, far = 0.0;
+        for (int a = 0; a < 3; ++a) {
+            extent = std::max(extent, ws_hi[a] - (double)t.ws_lo[a]);
+            far = std::max({far, std::fabs((double)t.ws_lo[a]), std::fabs(ws_hi[a])});
+        }
+        t.pq = (float)std::min(61440.0 / extent, far > 0.0 ? 1e10 / far : HUGE_VAL);
+        for (int a = 0; a < 3; ++a)
+            t.pc[a] = (float)((double)kFieldMagic + 2048.0 - (double)t.ws_lo[a] * (double)t.pq);
+    }
     // the distance field and the links' thresholds in its unit
     float edge = 0.f, shrink = 0.f;
     bool build = false;

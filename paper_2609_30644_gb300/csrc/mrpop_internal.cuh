@@ -42,6 +42,10 @@ struct Tables {
     // 1 m): coordinates taken relative to it are >= 0, so their float bits
     // order like unsigned integers.
     float ws_lo[3] = {0.f, 0.f, 0.f};
+    // Grid coordinates of the robot-robot culling levels: fmaf(x, pq, pc[axis])
+    // rounds a coordinate of a coarse centre to a whole number of steps of
+    // 1 / pq in its low 16 mantissa bits (kFieldMagic's scheme).
+    float pq = 0.f, pc[3] = {0.f, 0.f, 0.f};
     // Distance field of the obstacles (DistanceField below).
     const uint8_t *df = nullptr;  // [df_n[2]][df_n[1]][df_n[0]], device
     int df_n[3] = {0, 0, 0};      // voxels per axis (0: none)
@@ -105,12 +109,13 @@ inline int validate_warp_floats(const Tables &t, int fine) {
 }
 
 // Per-warp shared scratch of the verdict body (floats): (q_a, q_b - q_a) of
-// every joint and a spare one, the robots' tile boxes and the coarse centres of
-// every link.
+// every joint and a spare one, the robots' tile boxes and every link's coarse
+// centres as 16-bit grid coordinates (three per lane), which halve the scratch
+// that limits the resident warps of many-arm scenes.
 inline int verdict_dpad(const Tables &t) { return (t.L + 4) & ~3; }
 inline int verdict_warp_floats(const Tables &t) {
     const int dpad = verdict_dpad(t);
-    return 2 * dpad + 8 * t.K + t.L * kXcFloats * 32;
+    return 2 * dpad + 8 * t.K + t.L * kXcFloats * 16;
 }
 
 struct DeviceProblem {

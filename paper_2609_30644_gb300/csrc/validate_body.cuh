@@ -720,25 +720,37 @@ __device__ __forceinline__ int interval_count(const float2 *ad, int D, float res
     return nf > 1073741824.f ? 1073741824 : (int)nf;
 }
 
+// A stored 16-bit grid coordinate as a float of kFieldMagic's scheme: differences
+// of two are whole steps, exactly.  Each is within half a step of its
+// coordinate, so a distance of two points in steps is within sqrt(3) of the
+// true one: kGridSlack.
+__device__ __forceinline__ float grid_float(unsigned v) {
+    return __uint_as_float((unsigned)kFieldMagicBits + v);
+}
+constexpr float kGridSlack = 2.f;
+
 // Fine robot-robot test of link l (frame F) against link i: true where a
 // sphere of one touches a sphere of the other at the lane's checkpoint.  Only
 // lanes whose own coarse spheres touch (own) can; each sphere of l is first
-// tested against i's coarse sphere (centre x, which encloses i's spheres with
-// slack), and i's spheres are placed when one of them is near.
+// tested against i's coarse sphere (grid coordinates x; it encloses i's spheres
+// with slack), and i's spheres are placed when one of them is near.
 __device__ __forceinline__ bool fine_pair(const float4 *tab, const Tables &t, const float2 *ad,
                                           float tk, const Frame &F, int l, int i,
-                                          bool own, const float *x, float m) {
+                                          bool own, const uint16_t *x, float m) {
     const float4 LBl = tab[t.off_link + kLinkF4 * l + 1], LBi = tab[t.off_link + kLinkF4 * i + 1];
     const int sf = __float_as_int(LBl.y), ns = __float_as_int(LBl.z);
     const int sfi = __float_as_int(LBi.y), nsi = __float_as_int(LBi.z);
+    const float pq = t.pq, pcx = t.pc[0], pcy = t.pc[1], pcz = t.pc[2];
     const float rci = tab[t.off_link + kLinkF4 * i + 2].w + m;
-    const float xi = x[0], yi = x[32], zi = x[64];
+    const float xi = grid_float(x[0]), yi = grid_float(x[32]), zi = grid_float(x[64]);
     unsigned near = 0;  // spheres of l near i's coarse sphere in some lane
     for (int s = 0; s < ns; ++s) {
         const float4 sp = tab[t.off_sph + sf + s];
         const float3 p = apply(F, sp.x, sp.y, sp.z);
-        const float th = sp.w + rci;
-        near |= own && dist2(p.x, p.y, p.z, xi, yi, zi) < th * th ? 1u << s : 0u;
+        const float th = fmaf(sp.w + rci, pq, kGridSlack);
+        near |= own && dist2(fmaf(p.x, pq, pcx), fmaf(p.y, pq, pcy), fmaf(p.z, pq, pcz), xi, yi, zi) <
+                           th * th
+                    ? 1u << s : 0u;
     }
     near = __reduce_or_sync(kFull, near);
     if (!near) return false;
@@ -772,17 +784,20 @@ __device__ __forceinline__ bool fine_pair(const float4 *tab, const Tables &t, co
 // lane's checkpoint, then the spheres of the pairs that some lane hit.
 __device__ __forceinline__ bool link_pairs(const float4 *tab, const Tables &t, const float2 *ad,
                                            float tk, int l, bool near, int first,
-                                           unsigned mask, const float *xc, float m) {
+                                           unsigned mask, const uint16_t *xc, float m) {
     const int lane = threadIdx.x & 31, o_link = t.off_link;
-    const float *x = xc + l * (kXcFloats * 32) + lane;
-    const float cx = x[0], cy = x[32], cz = x[64], rl = tab[o_link + kLinkF4 * l + 2].w;
+    const uint16_t *x = xc + l * (kXcFloats * 32) + lane;
+    const float cx = grid_float(x[0]), cy = grid_float(x[32]), cz = grid_float(x[64]);
+    const float rl = tab[o_link + kLinkF4 * l + 2].w + m, pq = t.pq;
     unsigned own = 0;
     for (unsigned mm = mask; mm; mm &= mm - 1) {
         const int bit = __ffs(mm) - 1, i = first + bit;
         if (__float_as_int(tab[o_link + kLinkF4 * i + 1].z) == 0) continue;  // no spheres
-        const float *y = xc + i * (kXcFloats * 32) + lane;
-        const float th2 = rl + tab[o_link + kLinkF4 * i + 2].w + m;
-        own |= near && dist2(cx, cy, cz, y[0], y[32], y[64]) < th2 * th2 ? 1u << bit : 0u;
+        const uint16_t *y = xc + i * (kXcFloats * 32) + lane;
+        const float th = fmaf(rl + tab[o_link + kLinkF4 * i + 2].w, pq, kGridSlack);
+        own |= near && dist2(cx, cy, cz, grid_float(y[0]), grid_float(y[32]), grid_float(y[64])) <
+                           th * th
+                   ? 1u << bit : 0u;
     }
     unsigned wi = __reduce_or_sync(kFull, own);
     if (!wi) return false;
@@ -937,8 +952,9 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
     float *ws = reinterpret_cast<float *>(sm4 + t.n_f4) + (size_t)warp * P.warp_floats;
     float2 *ad = reinterpret_cast<float2 *>(ws);  // (q_a, q_b - q_a) of each joint, one spare
     const int dpad = (D + 4) & ~3;                             // verdict_dpad
-    float4 *rb = reinterpret_cast<float4 *>(ws + 2 * dpad);    // robot tile boxes [K][2]
-    float *xc = ws + 2 * dpad + 8 * K;                         // coarse centres [L][3][32]
+    int4 *rb = reinterpret_cast<int4 *>(ws + 2 * dpad);        // robot tile boxes [K][2]
+    // coarse centres in grid coordinates [L][3][32]
+    uint16_t *xc = reinterpret_cast<uint16_t *>(ws + 2 * dpad + 8 * K);
 
     for (int i = threadIdx.x; i < t.n_f4; i += blockDim.x) tab[i] = P.blob[i];
     __syncthreads();
@@ -949,6 +965,7 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
     const float fi = t.df_inv, fx = t.df_c[0], fy = t.df_c[1], fz = t.df_c[2];
     const unsigned fnx = t.df_n[0], fny = t.df_n[1], fnz = t.df_n[2];
     const int fout = t.df_out;
+    const float pq = t.pq, pcx = t.pc[0], pcy = t.pc[1], pcz = t.pc[2];
     const float m = P.margin;
     if (lane == 0) ad[D] = make_float2(0.f, 0.f);
     const bool pairs = K > 1 || t.selfcol;
@@ -996,10 +1013,10 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
             for (int b = 0; b < K && !edge_hit; ++b) {
                 const int l0 = t.link0[b], l1 = t.link0[b + 1];
                 Frame Tm = load_base(tab, t, b);
-                float bx0 = FLT_MAX, by0 = FLT_MAX, bz0 = FLT_MAX;  // box of the lane's centres
-                float bx1 = -FLT_MAX, by1 = -FLT_MAX, bz1 = -FLT_MAX;
+                // box of the lane's centres (float bits, positive: ordered)
+                unsigned bx0 = kFull, by0 = kFull, bz0 = kFull, bx1 = 0, by1 = 0, bz1 = 0;
                 const float4 *lk = tab + o_link + kLinkF4 * l0;
-                float *x = xc + l0 * (kXcFloats * 32) + lane;
+                uint16_t *x = xc + l0 * (kXcFloats * 32) + lane;
                 const float2 *aj = ad + l0 + 1;  // the next link's joint
                 const float rmax = lk[3].y;  // the robot's largest coarse radius, -1: no spheres
                 bool hit = false;
@@ -1021,16 +1038,19 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
                     const float2 qd = *aj++;
                     joint_sincos(__fmaf_rn(tk, qd.y, qd.x) + LD.z, &sn, &cs);
                     if (pairs) {
-                        x[0] = cc.x;
-                        x[32] = cc.y;
-                        x[64] = cc.z;
+                        const unsigned gx = __float_as_uint(fmaf(cc.x, pq, pcx));
+                        const unsigned gy = __float_as_uint(fmaf(cc.y, pq, pcy));
+                        const unsigned gz = __float_as_uint(fmaf(cc.z, pq, pcz));
+                        x[0] = (uint16_t)gx;
+                        x[32] = (uint16_t)gy;
+                        x[64] = (uint16_t)gz;
                         // (a link without spheres only widens the box)
-                        bx0 = fminf(bx0, cc.x);
-                        bx1 = fmaxf(bx1, cc.x);
-                        by0 = fminf(by0, cc.y);
-                        by1 = fmaxf(by1, cc.y);
-                        bz0 = fminf(bz0, cc.z);
-                        bz1 = fmaxf(bz1, cc.z);
+                        bx0 = min(bx0, gx);
+                        bx1 = max(bx1, gx);
+                        by0 = min(by0, gy);
+                        by1 = max(by1, gy);
+                        bz0 = min(bz0, gz);
+                        bz1 = max(bz1, gz);
                     }
                     const bool near = v < th;
                     if (__any_sync(kFull, near)) {
@@ -1044,22 +1064,20 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
                     x += kXcFloats * 32;
                 }
                 if (edge_hit || rmax < 0.f) {
-                    if (lane == 0) rb[2 * b].w = -1.f;  // no spheres: pairs with nothing
+                    if (lane == 0) rb[2 * b].w = __float_as_int(-1.f);  // no spheres: pairs with nothing
                     continue;
                 }
                 if (K > 1) {
-                    // the robot's box over the tile, relative to the workspace
-                    // corner as the tile bounds are
-                    const float wlx = t.ws_lo[0], wly = t.ws_lo[1], wlz = t.ws_lo[2];
-                    float4 lo, hi;
-                    lo.x = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(bx0 - wlx)));
-                    hi.x = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(bx1 - wlx)));
-                    lo.y = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(by0 - wly)));
-                    hi.y = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(by1 - wly)));
-                    lo.z = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(bz0 - wlz)));
-                    hi.z = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(bz1 - wlz)));
-                    lo.w = rmax;
-                    hi.w = 0.f;
+                    // the robot's box over the tile
+                    int4 lo, hi;
+                    lo.x = (int)__reduce_min_sync(kFull, bx0);
+                    hi.x = (int)__reduce_max_sync(kFull, bx1);
+                    lo.y = (int)__reduce_min_sync(kFull, by0);
+                    hi.y = (int)__reduce_max_sync(kFull, by1);
+                    lo.z = (int)__reduce_min_sync(kFull, bz0);
+                    hi.z = (int)__reduce_max_sync(kFull, bz1);
+                    lo.w = __float_as_int(rmax);
+                    hi.w = 0;
                     if (lane == 0) {
                         rb[2 * b] = lo;
                         rb[2 * b + 1] = hi;
@@ -1067,38 +1085,42 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
                     __syncwarp();
                     bool close = false;
                     if (lane < b) {
-                        const float4 ol = rb[2 * lane], oh = rb[2 * lane + 1];
-                        const float gx = fmaxf(fmaxf(ol.x - hi.x, lo.x - oh.x), 0.f);
-                        const float gy = fmaxf(fmaxf(ol.y - hi.y, lo.y - oh.y), 0.f);
-                        const float gz = fmaxf(fmaxf(ol.z - hi.z, lo.z - oh.z), 0.f);
-                        const float r = ol.w + rmax + m + kTileSlack;
-                        close = ol.w >= 0.f && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < r * r;
+                        const int4 ol = rb[2 * lane], oh = rb[2 * lane + 1];
+                        const float gx = (float)max(max(ol.x - hi.x, lo.x - oh.x), 0);
+                        const float gy = (float)max(max(ol.y - hi.y, lo.y - oh.y), 0);
+                        const float gz = (float)max(max(ol.z - hi.z, lo.z - oh.z), 0);
+                        const float ro = __int_as_float(ol.w);
+                        const float r = fmaf(ro + rmax + m + kTileSlack, pq, kGridSlack);
+                        close = ro >= 0.f && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < r * r;
                     }
                     for (unsigned cm = __ballot_sync(kFull, close); cm; cm &= cm - 1) {
                         const int a = __ffs(cm) - 1;
                         const int a0 = t.link0[a], a1 = t.link0[a + 1];
                         // robot a's box at the lane's checkpoint
-                        float ax0 = FLT_MAX, ay0 = FLT_MAX, az0 = FLT_MAX;
-                        float ax1 = -FLT_MAX, ay1 = -FLT_MAX, az1 = -FLT_MAX;
+                        unsigned ux0 = kFull, uy0 = kFull, uz0 = kFull, ux1 = 0, uy1 = 0, uz1 = 0;
                         for (int i = a0; i < a1; ++i) {
-                            if (__float_as_int(tab[o_link + kLinkF4 * i + 3].x) == 0) continue;
-                            const float *x = xc + i * (kXcFloats * 32) + lane;
-                            ax0 = fminf(ax0, x[0]);
-                            ax1 = fmaxf(ax1, x[0]);
-                            ay0 = fminf(ay0, x[32]);
-                            ay1 = fmaxf(ay1, x[32]);
-                            az0 = fminf(az0, x[64]);
-                            az1 = fmaxf(az1, x[64]);
+                            const uint16_t *x = xc + i * (kXcFloats * 32) + lane;
+                            const unsigned vx = x[0], vy = x[32], vz = x[64];
+                            ux0 = min(ux0, vx);
+                            ux1 = max(ux1, vx);
+                            uy0 = min(uy0, vy);
+                            uy1 = max(uy1, vy);
+                            uz0 = min(uz0, vz);
+                            uz1 = max(uz1, vz);
                         }
-                        const float ra = rb[2 * a].w + m + kTileSlack;
+                        const float ax0 = grid_float(ux0), ay0 = grid_float(uy0), az0 = grid_float(uz0);
+                        const float ax1 = grid_float(ux1), ay1 = grid_float(uy1), az1 = grid_float(uz1);
+                        const float ra = __int_as_float(rb[2 * a].w) + m + kTileSlack;
                         unsigned nl = 0;
                         for (int l = l0; l < l1; ++l) {
                             if (__float_as_int(tab[o_link + kLinkF4 * l + 3].x) == 0) continue;
-                            const float *x = xc + l * (kXcFloats * 32) + lane;
-                            const float gx = fmaxf(fmaxf(ax0 - x[0], x[0] - ax1), 0.f);
-                            const float gy = fmaxf(fmaxf(ay0 - x[32], x[32] - ay1), 0.f);
-                            const float gz = fmaxf(fmaxf(az0 - x[64], x[64] - az1), 0.f);
-                            const float r = tab[o_link + kLinkF4 * l + 2].w + ra;
+                            const uint16_t *x = xc + l * (kXcFloats * 32) + lane;
+                            const float vx = grid_float(x[0]), vy = grid_float(x[32]),
+                                        vz = grid_float(x[64]);
+                            const float gx = fmaxf(fmaxf(ax0 - vx, vx - ax1), 0.f);
+                            const float gy = fmaxf(fmaxf(ay0 - vy, vy - ay1), 0.f);
+                            const float gz = fmaxf(fmaxf(az0 - vz, vz - az1), 0.f);
+                            const float r = fmaf(tab[o_link + kLinkF4 * l + 2].w + ra, pq, kGridSlack);
                             nl |= fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < r * r ? 1u << (l - l0) : 0u;
                         }
                         for (unsigned wl = __reduce_or_sync(kFull, nl); wl; wl &= wl - 1) {

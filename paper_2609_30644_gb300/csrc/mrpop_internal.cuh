@@ -108,14 +108,15 @@ inline int validate_warp_floats(const Tables &t, int fine) {
     return 2 * dpad + 4 * nstore + nstore * kXcFloats * 32 + (fine ? kFrFloats * 32 + 64 : 0);
 }
 
-// Per-warp shared scratch of the verdict body (floats): (q_a, q_b - q_a) of
+// Per-warp shared scratch of the verdict body (floats): the warp's edge (8
+// words), (q_a, q_b - q_a) of
 // every joint and a spare one, the robots' tile boxes and every link's coarse
 // centres as 16-bit grid coordinates (three per lane), which halve the scratch
 // that limits the resident warps of many-arm scenes.
 inline int verdict_dpad(const Tables &t) { return (t.L + 4) & ~3; }
 inline int verdict_warp_floats(const Tables &t) {
     const int dpad = verdict_dpad(t);
-    return 2 * dpad + 8 * t.K + t.L * kXcFloats * 16;
+    return 8 + 2 * dpad + 8 * t.K + t.L * kXcFloats * 16;
 }
 
 struct DeviceProblem {

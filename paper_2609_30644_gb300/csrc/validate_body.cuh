@@ -927,10 +927,17 @@ __device__ __forceinline__ bool link_obstacles(const float4 *tab, const Tables &
 // bound (six warp reductions) and tested it against all obstacles and earlier
 // links, about 230 of the 279 instructions a link took; an eighth of the links
 // now needs any of that (65,536 candidate edges of the table pair: 312 M
-// instructions and 324 us before, 204 M and 240 us now; 8 arms, 4,099 edges: 57
-// M and 480 us, 32 M and 258 us).  Running all of a robot's links first and
+// instructions and 324 us before, 223 M and 245 us now; 8 arms, 4,099 edges:
+// 57 M and 480 us, 32 M and 176 us).  Running all of a robot's links first and
 // rebuilding the near ones' frames afterwards was slower (292 us: more joints
 // before a colliding link ends the edge).
+//
+// A warp that finds no edge left takes tiles of the edges that the block's
+// other warps still work on: an edge's tiles are claimed one by one from its
+// owner's words in shared memory, the first hit writes the verdict 0 and the
+// warp that completes the last tile without one writes 1, so nobody waits.
+// Without it a launch or a planner chunk ends with its longest edges, one warp
+// each (8 arms, 4,099 edges: 256 us, with it 176).
 //
 // LOCAL: the edges [e0, e1) are handed out to the block's warps through the
 // shared-memory counter *s_next (zeroed by the caller before the call) instead
@@ -942,6 +949,20 @@ __device__ __forceinline__ bool link_obstacles(const float4 *tab, const Tables &
 // another.  The caller gives a shared flag (zero) in s_next.  With LOCAL too, the
 // warps of each of the edges [e0, e1) are (P.warps / their number) in a row, s_next
 // holds a zero flag for each, and the caller turns the flags into verdicts.
+struct EdgeWords {
+    // the owner's edge count (high half) and the next tile to claim (low half),
+    // kClosed while the words below and the owner's joints are being written:
+    // a claim is a compare-and-swap, so it only succeeds on the edge whose
+    // words were read under the same count
+    unsigned claim;
+    int e, n;   // the edge and its interval count
+    int T;      // its tiles
+    int done;   // tiles completed without a hit
+    int hit;
+    int pad[2];
+};
+constexpr unsigned kClosed = 0xffffu;  // above any tile (32,769 at most)
+
 template <bool LOCAL, bool GROUP = false>
 __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int e0 = 0, int e1 = 0,
                                              int *s_next = nullptr) {
@@ -949,14 +970,19 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Tables &t = P.t;
     const int K = t.K, D = t.L;
-    float *ws = reinterpret_cast<float *>(sm4 + t.n_f4) + (size_t)warp * P.warp_floats;
+    float *ws_all = reinterpret_cast<float *>(sm4 + t.n_f4);
+    float *ws = ws_all + (size_t)warp * P.warp_floats + 8;
     float2 *ad = reinterpret_cast<float2 *>(ws);  // (q_a, q_b - q_a) of each joint, one spare
+    auto words = [&](int w) {
+        return reinterpret_cast<EdgeWords *>(ws_all + (size_t)w * P.warp_floats);
+    };
     const int dpad = (D + 4) & ~3;                             // verdict_dpad
     int4 *rb = reinterpret_cast<int4 *>(ws + 2 * dpad);        // robot tile boxes [K][2]
     // coarse centres in grid coordinates [L][3][32]
     uint16_t *xc = reinterpret_cast<uint16_t *>(ws + 2 * dpad + 8 * K);
 
     for (int i = threadIdx.x; i < t.n_f4; i += blockDim.x) tab[i] = P.blob[i];
+    if (!GROUP && lane == 0 && warp < P.warps) words(warp)->claim = kClosed;
     __syncthreads();
     if (warp >= P.warps) return;  // spare warps of a shared multi-problem launch
 
@@ -970,38 +996,125 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
     if (lane == 0) ad[D] = make_float2(0.f, 0.f);
     const bool pairs = K > 1 || t.selfcol;
     const int split = GROUP ? (LOCAL ? P.warps / max(e1 - e0, 1) : P.warps) : 1;  // warps per edge
+    int helping = 0;  // other warps looked at since the last edge (0: owner)
     for (;;) {
-        int e = 0;
-        if (GROUP && LOCAL) {
-            e = e0 + warp / split;
-            if (e >= e1) return;
-        } else if (GROUP) {
-            e = blockIdx.x;
+        int e = 0, n = 0, T = 0;
+        bool edge_hit = false;
+        EdgeWords *ew = words(warp);
+        unsigned seen = 0;  // a helper's view of the owner's claim word
+        if (GROUP || helping == 0) {
+            if (GROUP && LOCAL) {
+                e = e0 + warp / split;
+                if (e >= e1) return;
+            } else if (GROUP) {
+                e = blockIdx.x;
+            } else {
+                if (lane == 0) e = LOCAL ? e0 + atomicAdd(s_next, 1) : atomicAdd(&P.work[0], 1);
+                e = __shfl_sync(kFull, e, 0);
+                if (e >= (LOCAL ? e1 : P.E)) {
+                    helping = 1;
+                    continue;
+                }
+            }
+            if (!GROUP && lane == 0) {
+                const unsigned c = *(volatile unsigned *)&ew->claim;
+                *(volatile unsigned *)&ew->claim = (c + 0x10000u) | kClosed;
+                __threadfence_block();
+            }
+            __syncwarp();
+            for (int i = lane; i < D; i += 32) {
+                // (the persistent planner rewrites its edge buffers within one
+                // launch: there the loads bypass the non-coherent cache)
+                const float a =
+                    LOCAL ? __ldcg(P.qa + (size_t)i * P.E + e) : __ldg(P.qa + (size_t)i * P.E + e);
+                const float b =
+                    LOCAL ? __ldcg(P.qb + (size_t)i * P.E + e) : __ldg(P.qb + (size_t)i * P.E + e);
+                ad[i] = make_float2(a, __fsub_rn(b, a));
+            }
+            __syncwarp();
+            float len;
+            n = interval_count(ad, D, P.res, &len);
+            // Edges beyond MRPOP_MAX_EDGE_INTERVALS intervals (or with non-finite
+            // coordinates) are reported invalid without being checked.
+            const bool too_long = !(len <= P.res * (float)MRPOP_MAX_EDGE_INTERVALS);
+            T = too_long ? 0 : (n >> 5) + 1;  // ceil((n + 1) / 32)
+            edge_hit = too_long;
+            if (lane == 0 && (!GROUP || !LOCAL)) {
+                if (P.length) P.length[e] = len;
+                if (P.npoints) P.npoints[e] = n;
+                if (!GROUP && too_long) P.valid[e] = 0;
+            }
+            if (!GROUP) {
+                if (too_long) continue;
+                if (T > 1 && lane == 0) {  // (a single tile is its owner's alone)
+                    ew->e = e;
+                    ew->n = n;
+                    ew->T = T;
+                    ew->done = ew->hit = 0;
+                    __threadfence_block();
+                    *(volatile unsigned *)&ew->claim &= ~0xffffu;  // open, tile 0 next
+                }
+                __syncwarp();
+            }
         } else {
-            if (lane == 0) e = LOCAL ? e0 + atomicAdd(s_next, 1) : atomicAdd(&P.work[0], 1);
-            e = __shfl_sync(kFull, e, 0);
-            if (e >= (LOCAL ? e1 : P.E)) break;
+            // no edge is left to fetch: an owner's open edge is its last, which
+            // it leaves only once every tile is claimed or one has hit
+            if (helping >= P.warps) break;
+            int w = warp + helping;
+            if (w >= P.warps) w -= P.warps;
+            ++helping;
+            ew = words(w);
+            int4 v = make_int4(0, 0, 0, 0);  // (one lane looks: the words may be changing)
+            if (lane == 0) {
+                const volatile EdgeWords *vw = ew;
+                v.x = (int)vw->claim;
+                __threadfence_block();
+                v.y = vw->T;
+                v.z = vw->e;
+                v.w = vw->n;
+                // closed, all claimed or hit: nothing to take
+                if ((v.x & 0xffff) >= v.y || (v.x & 0xffff) == (int)kClosed || vw->hit) v.y = 0;
+            }
+            T = __shfl_sync(kFull, v.y, 0);
+            if (T == 0) continue;
+            seen = (unsigned)__shfl_sync(kFull, v.x, 0);
+            e = __shfl_sync(kFull, v.z, 0);
+            n = __shfl_sync(kFull, v.w, 0);
+            const float2 *from = reinterpret_cast<const float2 *>(ew + 1);
+            __syncwarp();
+            for (int i = lane; i < D; i += 32) ad[i] = from[i];
+            __syncwarp();
         }
-        __syncwarp();
-        for (int i = lane; i < D; i += 32) {
-            // (the persistent planner rewrites its edge buffers within one
-            // launch: there the loads bypass the non-coherent cache)
-            const float a = LOCAL ? __ldcg(P.qa + (size_t)i * P.E + e) : __ldg(P.qa + (size_t)i * P.E + e);
-            const float b = LOCAL ? __ldcg(P.qb + (size_t)i * P.E + e) : __ldg(P.qb + (size_t)i * P.E + e);
-            ad[i] = make_float2(a, __fsub_rn(b, a));
-        }
-        __syncwarp();
-        float len;
-        const int n = interval_count(ad, D, P.res, &len);
-        // Edges beyond MRPOP_MAX_EDGE_INTERVALS intervals (or with non-finite
-        // coordinates) are reported invalid without being checked.
-        const bool too_long = !(len <= P.res * (float)MRPOP_MAX_EDGE_INTERVALS);
-        const int T = too_long ? 0 : (n >> 5) + 1;  // ceil((n + 1) / 32)
-        bool edge_hit = too_long;
 
         volatile int *flag = GROUP ? s_next + (LOCAL ? e - e0 : 0) : nullptr;
-        for (int tile = GROUP ? warp % split : 0; tile < T && !edge_hit; tile += split) {
-            if (GROUP && *flag) break;  // another warp's tile collides
+        for (int own = GROUP ? warp % split : 0;; own += split) {
+            int tile = own;
+            if (GROUP) {
+                if (tile >= T || edge_hit || *flag) break;  // (another warp's tile collides)
+            } else if (T > 1) {
+                if (lane == 0) {
+                    tile = T;
+                    if (!*(volatile int *)&ew->hit) {
+                        if (helping == 0) {
+                            tile = (int)(atomicAdd(&ew->claim, 1u) & 0xffffu);
+                        } else {
+                            __threadfence_block();
+                            unsigned c = *(volatile unsigned *)&ew->claim;
+                            while ((c >> 16) == (seen >> 16) && (int)(c & 0xffffu) < T) {
+                                const unsigned got = atomicCAS(&ew->claim, c, c + 1u);
+                                if (got == c) {
+                                    tile = (int)(c & 0xffffu);
+                                    break;
+                                }
+                                c = got;
+                            }
+                        }
+                    }
+                }
+                tile = __shfl_sync(kFull, tile, 0);
+                if (tile >= T) break;
+                if (helping) helping = 1;  // look at every warp again afterwards
+            }
             int k = P.order ? tile * 32 + lane : tile + T * lane;
             k = min(k, n);
             // (k = 0 apart: a zero numerator sends the whole warp through the
@@ -1144,19 +1257,27 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
                         edge_hit = __any_sync(kFull, hit);
                     }
             }
+            if (!GROUP) {
+                if (lane == 0) {
+                    if (T == 1) {
+                        P.valid[e] = edge_hit ? 0 : 1;
+                    } else if (edge_hit) {
+                        *(volatile int *)&ew->hit = 1;
+                        P.valid[e] = 0;
+                    } else if (atomicAdd(&ew->done, 1) == T - 1) {
+                        P.valid[e] = 1;
+                    }
+                }
+                if (edge_hit || tile == T - 1) break;  // (every tile is claimed)
+            }
         }
         if (GROUP) {
             if (lane == 0 && edge_hit) *flag = 1;
             if (LOCAL) return;
             __syncthreads();
-            edge_hit = *flag != 0;
+            if (threadIdx.x == 0) P.valid[e] = *flag == 0;
+            return;
         }
-        if (lane == 0 && (!GROUP || warp == 0)) {
-            P.valid[e] = edge_hit ? 0 : 1;
-            if (P.length) P.length[e] = len;
-            if (P.npoints) P.npoints[e] = n;
-        }
-        if (GROUP) return;
     }
     // The last warp to leave resets the work counter for the next launch on
     // this problem (every warp has made its final fetch before counting out).

@@ -1115,11 +1115,10 @@ def run_ours(args) -> None:
             "clocks": clk,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(h2d),
                     "d2h_bytes_per_step": int(d2h)},
-            # per step: validate; NEAREST = setup (+ g range), histogram (+
+            # per step: validate; NEAREST = setup (bucket limits), histogram (+
             # scan), scatter, seeding (+ cuts) and the FP32 filter kernel (+
-            # reduce); neighbors over vertex ranges + the ordered merge; path
-            # cost + its sum
-            "gpu_launches": 10 * args.steps,
+            # reduce); NEIGHBORS and path cost one cluster launch each
+            "gpu_launches": 8 * args.steps,
             "cpu_baseline": cpu,
             "planner": planner,
             "serving": serving,

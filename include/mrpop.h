@@ -182,9 +182,11 @@ mrpop_status mrpop_validate_edges_ex(mrpop_problem *p, const float *qa, const fl
 mrpop_status mrpop_edge_clearance(mrpop_problem *p, const float *qa, const float *qb,
                                   int64_t n_edges, float *min_clear, void *cuda_stream);
 
-/* Work counters of mrpop_validate_edges on the same inputs, summed over the
- * batch, for roofline accounting (device int64 [MRPOP_WORK_COUNTERS],
- * overwritten):
+/* Work counters of validating the same inputs, summed over the batch, for
+ * roofline accounting (device int64 [MRPOP_WORK_COUNTERS], overwritten).  They
+ * describe the culling hierarchy from the tile bounds down;
+ * mrpop_validate_edges also holds a distance field of the obstacles and skips
+ * what the field clears, so it does less:
  *   [0]  checkpoints evaluated             [1]  joint transforms
  *   [2]  checkpoint link-vs-obstacle-sphere bound tests (tile candidates only)
  *   [3]  checkpoint link-vs-link bound tests (tile candidates only)

@@ -230,13 +230,9 @@ __device__ __forceinline__ int interval_count(const float *dq, int D, float res,
 // encloses what it replaces with at least 1e-4 m of slack), so the minimum is
 // that over all pairs, to the bit.  Measuring every pair, with a square root
 // each, took 2,929 us for 1,023 edges of the table pair; this takes 90 us.
-//
-// LOCAL: the edges [e0, e1) are handed out to the block's warps through the
-// shared-memory counter *s_next (zeroed by the caller before the call) instead
-// of the problem's global work counter, which is then left untouched.
-template <int MODE, bool RA, bool LOCAL = false>
-__device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int e0 = 0,
-                                              int e1 = 0, int *s_next = nullptr) {
+template <int MODE, bool RA>
+__device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4) {
+    static_assert(MODE != kVerdict || RA, "plain verdicts take verdict_body");
     float4 *tab = sm4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float *ws = reinterpret_cast<float *>(sm4 + P.t.n_f4) + (size_t)warp * P.warp_floats;
@@ -263,15 +259,13 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
 
     for (;;) {
         int e = 0;
-        if (lane == 0) e = LOCAL ? e0 + atomicAdd(s_next, 1) : atomicAdd(&P.work[0], 1);
+        if (lane == 0) e = atomicAdd(&P.work[0], 1);
         e = __shfl_sync(kFull, e, 0);
-        if (e >= (LOCAL ? e1 : P.E)) break;
+        if (e >= P.E) break;
         __syncwarp();
         for (int i = lane; i < D; i += 32) {
-            // (the persistent planner rewrites its edge buffers within one
-            // launch: there the loads bypass the non-coherent cache)
-            const float a = LOCAL ? __ldcg(P.qa + (size_t)i * P.E + e) : __ldg(P.qa + (size_t)i * P.E + e);
-            const float b = LOCAL ? __ldcg(P.qb + (size_t)i * P.E + e) : __ldg(P.qb + (size_t)i * P.E + e);
+            const float a = __ldg(P.qa + (size_t)i * P.E + e);
+            const float b = __ldg(P.qb + (size_t)i * P.E + e);
             qa_s[i] = a;
             dq_s[i] = __fsub_rn(b, a);
         }
@@ -685,7 +679,7 @@ __device__ __forceinline__ void validate_body(const VParams &P, float4 *sm4, int
     }
     // The last warp to leave resets the work counter for the next launch on
     // this problem (every warp has made its final fetch before counting out).
-    if (!LOCAL && lane == 0) {
+    if (lane == 0) {
         __threadfence();
         if (atomicAdd(&P.work[1], 1) == P.total_warps - 1) {
             atomicExch(&P.work[0], 0);

@@ -2325,11 +2325,12 @@ constexpr int kPathThreads = 512;
 // Each block sums the segments [block * chunk, block * chunk + chunk) in a
 // fixed order (per thread in steps of the block, then a tree in shared memory:
 // FP64 additions are scarce, so no warp repeats another's).  A cluster of up to
-// 8 blocks covers a path of up to 131,072 segments and its first block adds the
-// blocks' sums in block order: one launch and no scratch, where the partial
-// sums' allocation, a second kernel and 4-byte loads took 20.4 to 22.8 us a call
-// for 65,537 vertices in 14-D (19.2 us now, most of it the host's).  Longer paths write their sums to partial,
-// which a second kernel adds.
+// 8 blocks covers a path of up to 16,384 segments and its first block adds the
+// blocks' sums in block order: one launch and no scratch (16,385 vertices in
+// 14-D: 12.3 us with a cold L2, 17.5 with 4-byte loads and a second kernel).
+// Longer paths need more SMs to read from memory (65,537 vertices in 14-D, cold:
+// 28.7 us as a cluster, 13.3 as 64 blocks; 131,073: 47 and 15.4): their blocks
+// write their sums to partial, which a second kernel adds.
 template <int V>
 __global__ void __launch_bounds__(kPathThreads)
 path_cost_kernel(const float *__restrict__ path, int64_t M, int dim, int64_t chunk,
@@ -2359,6 +2360,10 @@ path_cost_kernel(const float *__restrict__ path, int64_t M, int dim, int64_t chu
     }
     if (partial) {
         if (t == 0) partial[blockIdx.x] = acc;
+        return;
+    }
+    if (gridDim.x == 1) {
+        if (t == 0) *out = acc;
         return;
     }
     namespace cg = cooperative_groups;
@@ -2604,7 +2609,7 @@ static mrpop_status path_cost_v(const float *path, int64_t M, int dim, double *o
                                 cudaStream_t st) {
     const int64_t segs = M > 1 ? M - 1 : 0;
     constexpr int64_t kBlockSegs = 2 * kPathThreads;
-    if (segs <= 131072) {
+    if (segs <= 16384) {
         int blocks = 1;
         while (blocks < 8 && blocks * kBlockSegs < segs) blocks *= 2;
         cudaLaunchAttribute at{};

@@ -160,3 +160,11 @@ def test_path_cost_sizes(mp, M, D):
         # FP32 segment lengths: (D + 3) roundings of 2^-24 each at most
         assert abs(got - ref) <= (D + 3) * 2.0 ** -24 * ref
         assert mp.path_cost(path).item() == got
+
+
+@pytest.mark.parametrize("M", [16384, 16385, 16386, 17000])
+def test_path_cost_cluster_limit(mp, M):
+    path = torch.from_numpy(np.random.default_rng(M).uniform(-2.9, 2.9, (M, 14)).astype(np.float32)).cuda()
+    got = mp.path_cost(path).item()
+    ref = (path[1:].double() - path[:-1].double()).norm(dim=1).sum().item()
+    assert abs(got - ref) <= 17 * 2.0 ** -24 * ref

@@ -50,12 +50,12 @@ namespace {
 
 using namespace vb;
 
-template <int MODE, bool RA>
+template <int MODE, bool RA, bool SHARE = true>
 __global__ void __launch_bounds__(kWarpsMax * 32, MODE == kVerdict && !RA ? 7 : 1)
 validate_kernel(const __grid_constant__ VParams P) {
     extern __shared__ float4 sm4[];
     if constexpr (MODE == kVerdict && !RA)
-        verdict_body<false>(P, sm4);
+        verdict_body<false, false, SHARE>(P, sm4);
     else
         validate_body<MODE, RA>(P, sm4);
 }
@@ -72,11 +72,11 @@ validate_group_kernel(const __grid_constant__ VParams P) {
 // The same kernel with a wide register budget (up to 128 registers: four
 // blocks of four warps per SM): fewer warps, no spills in the robot-robot
 // fine stage, which many-arm scenes reach often.  An autotuner dimension.
-template <int MODE, bool RA>
+template <int MODE, bool RA, bool SHARE = true>
 __global__ void __launch_bounds__(kWarpsMax * 32, 4) validate_kernel_wide(const __grid_constant__ VParams P) {
     extern __shared__ float4 sm4[];
     if constexpr (MODE == kVerdict && !RA)
-        verdict_body<false>(P, sm4);
+        verdict_body<false, false, SHARE>(P, sm4);
     else
         validate_body<MODE, RA>(P, sm4);
 }
@@ -125,6 +125,20 @@ static mrpop_status cached_occupancy(const void *kern, int device, int smem_opti
     return MRPOP_OK;
 }
 
+// An edge per block, whose warps share its tiles, for up to kGroupWaves times
+// the edges whose blocks fit on the chip at once (table pair: 1,500 edges 33.8
+// us with an edge per warp, 26.5 so; 3,000 edges 39.9 and 42.6).
+constexpr int64_t kGroupWaves = 2;
+// Above that a warp takes an edge, and warps that find none left help the
+// others (SHARE), unless the claims cost more than the tail that they shorten:
+// with few links, whose tiles are short (planar pair, 6 links: 8,000 edges 35.4
+// us shared, 33.6 not; 65,536 edges 165 and 140), and with many edges for each
+// resident warp (table pair, 14 links, 4,256 warps: 8,000 edges 56 us shared,
+// 66 not; 16,000 edges 80 and 83; 32,768 edges 136 and 134; 65,536 edges 247
+// and 237).
+constexpr int kShareLinks = 10;
+constexpr int64_t kShareWaves = 6;
+
 template <int MODE, bool RA>
 mrpop_status launch_mode(mrpop_problem *p, VParams &V, int warps, size_t smem,
                          cudaStream_t st) {
@@ -135,15 +149,13 @@ mrpop_status launch_mode(mrpop_problem *p, VParams &V, int warps, size_t smem,
                                              warps * 32, smem, &bps);
     if (os != MRPOP_OK) return os;
     if (bps < 1) return set_error(MRPOP_EINVAL, "validation kernel does not fit on an SM");
-    // as many blocks as edges fit on the chip at once: an edge per block, whose
-    // warps share its tiles (256 planar edges, kernel: 18.6 us with an edge per
-    // warp, 13.4 us)
-    if (MODE == kVerdict && !RA && warps > 1 && V.E <= (int64_t)p->num_sms * bps) {
+    // few edges: 256 planar edges took 18.6 us with an edge per warp, 13.4 us here
+    if (MODE == kVerdict && !RA && warps > 1 && V.E <= kGroupWaves * p->num_sms * bps) {
         int gbps = 0;
         const mrpop_status gs = cached_occupancy((const void *)validate_group_kernel, p->device,
                                                  (int)p->smem_optin, warps * 32, smem, &gbps);
         if (gs != MRPOP_OK) return gs;
-        if (V.E <= (int64_t)p->num_sms * gbps) {
+        if (V.E <= kGroupWaves * p->num_sms * gbps) {
             V.warps = warps;
             validate_group_kernel<<<(int)V.E, warps * 32, smem, st>>>(V);
             MRPOP_CUDA_TRY(cudaGetLastError());
@@ -154,6 +166,11 @@ mrpop_status launch_mode(mrpop_problem *p, VParams &V, int warps, size_t smem,
     const int grid = (int)std::min<int64_t>((int64_t)p->num_sms * bps, want);
     V.total_warps = grid * warps;
     V.warps = warps;
+    if constexpr (MODE == kVerdict && !RA) {
+        if (V.t.L < kShareLinks || V.E > kShareWaves * V.total_warps)
+            kern = p->tuned_regs ? validate_kernel_wide<MODE, RA, false>
+                                 : validate_kernel<MODE, RA, false>;
+    }
     kern<<<grid, warps * 32, smem, st>>>(V);
     MRPOP_CUDA_TRY(cudaGetLastError());
     return MRPOP_OK;

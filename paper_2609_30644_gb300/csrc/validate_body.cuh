@@ -921,12 +921,12 @@ __device__ __forceinline__ bool link_obstacles(const float4 *tab, const Tables &
 // bound (six warp reductions) and tested it against all obstacles and earlier
 // links, about 230 of the 279 instructions a link took; an eighth of the links
 // now needs any of that (65,536 candidate edges of the table pair: 312 M
-// instructions and 324 us before, 223 M and 245 us now; 8 arms, 4,099 edges:
+// instructions and 324 us before, 204 M and 237 us now; 8 arms, 4,099 edges:
 // 57 M and 480 us, 32 M and 176 us).  Running all of a robot's links first and
 // rebuilding the near ones' frames afterwards was slower (292 us: more joints
 // before a colliding link ends the edge).
 //
-// A warp that finds no edge left takes tiles of the edges that the block's
+// SHARE: a warp that finds no edge left takes tiles of the edges that the block's
 // other warps still work on: an edge's tiles are claimed one by one from its
 // owner's words in shared memory, the first hit writes the verdict 0 and the
 // warp that completes the last tile without one writes 1, so nobody waits.
@@ -957,7 +957,7 @@ struct EdgeWords {
 };
 constexpr unsigned kClosed = 0xffffu;  // above any tile (32,769 at most)
 
-template <bool LOCAL, bool GROUP = false>
+template <bool LOCAL, bool GROUP = false, bool SHARE = !GROUP>
 __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int e0 = 0, int e1 = 0,
                                              int *s_next = nullptr) {
     float4 *tab = sm4;
@@ -976,7 +976,7 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
     uint16_t *xc = reinterpret_cast<uint16_t *>(ws + 2 * dpad + 8 * K);
 
     for (int i = threadIdx.x; i < t.n_f4; i += blockDim.x) tab[i] = P.blob[i];
-    if (!GROUP && lane == 0 && warp < P.warps) words(warp)->claim = kClosed;
+    if (SHARE && lane == 0 && warp < P.warps) words(warp)->claim = kClosed;
     __syncthreads();
     if (warp >= P.warps) return;  // spare warps of a shared multi-problem launch
 
@@ -996,7 +996,7 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
         bool edge_hit = false;
         EdgeWords *ew = words(warp);
         unsigned seen = 0;  // a helper's view of the owner's claim word
-        if (GROUP || helping == 0) {
+        if (!SHARE || helping == 0) {
             if (GROUP && LOCAL) {
                 e = e0 + warp / split;
                 if (e >= e1) return;
@@ -1006,11 +1006,12 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
                 if (lane == 0) e = LOCAL ? e0 + atomicAdd(s_next, 1) : atomicAdd(&P.work[0], 1);
                 e = __shfl_sync(kFull, e, 0);
                 if (e >= (LOCAL ? e1 : P.E)) {
+                    if (!SHARE) break;
                     helping = 1;
                     continue;
                 }
             }
-            if (!GROUP && lane == 0) {
+            if (SHARE && lane == 0) {
                 const unsigned c = *(volatile unsigned *)&ew->claim;
                 *(volatile unsigned *)&ew->claim = (c + 0x10000u) | kClosed;
                 __threadfence_block();
@@ -1036,9 +1037,9 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
             if (lane == 0 && (!GROUP || !LOCAL)) {
                 if (P.length) P.length[e] = len;
                 if (P.npoints) P.npoints[e] = n;
-                if (!GROUP && too_long) P.valid[e] = 0;
+                if (SHARE && too_long) P.valid[e] = 0;
             }
-            if (!GROUP) {
+            if (SHARE) {
                 if (too_long) continue;
                 if (T > 1 && lane == 0) {  // (a single tile is its owner's alone)
                     ew->e = e;
@@ -1083,8 +1084,9 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
         volatile int *flag = GROUP ? s_next + (LOCAL ? e - e0 : 0) : nullptr;
         for (int own = GROUP ? warp % split : 0;; own += split) {
             int tile = own;
-            if (GROUP) {
-                if (tile >= T || edge_hit || *flag) break;  // (another warp's tile collides)
+            if (!SHARE) {
+                if (tile >= T || edge_hit) break;
+                if (GROUP && *flag) break;  // another warp's tile collides
             } else if (T > 1) {
                 if (lane == 0) {
                     tile = T;
@@ -1251,7 +1253,7 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
                         edge_hit = __any_sync(kFull, hit);
                     }
             }
-            if (!GROUP) {
+            if (SHARE) {
                 if (lane == 0) {
                     if (T == 1) {
                         P.valid[e] = edge_hit ? 0 : 1;
@@ -1272,6 +1274,7 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
             if (threadIdx.x == 0) P.valid[e] = *flag == 0;
             return;
         }
+        if (!SHARE && lane == 0) P.valid[e] = edge_hit ? 0 : 1;
     }
     // The last warp to leave resets the work counter for the next launch on
     // this problem (every warp has made its final fetch before counting out).

@@ -108,3 +108,20 @@ def test_verdict_is_clearance_at_margin(mp, kind, n, self_collision, margin):
         d = (qb - qa).double().norm(dim=0)
         ok = torch.isfinite(d)
         torch.testing.assert_close(length.double()[ok], d[ok], rtol=1e-6, atol=1e-7)
+
+
+@pytest.mark.parametrize("kind,n,chunks", [
+    ("planar", 20000, (300, 1500, 4000)), ("table", 30000, (700, 1900, 2300, 9000))])
+def test_verdicts_do_not_depend_on_the_batch(mp, kind, n, chunks):
+    """An edge's verdict is the same in a batch that gives each warp many edges,
+    in one whose idle warps help and with a block to an edge."""
+    scene = _scene(kind)
+    qa, qb = synth.candidate_edges(scene, n, seed=5, step_hi=2.0)
+    qa, qb = torch.from_numpy(qa).cuda(), torch.from_numpy(qb).cuda()
+    with mp.Problem(scene, margin=1e-4) as p:
+        whole = mp.validate_edges(p, qa, qb).cpu()
+        assert 0 < int(whole.sum()) < n
+        for c in chunks:
+            for e0 in range(0, 3 * c, c):
+                a, b = (x[:, e0:e0 + c].contiguous() for x in (qa, qb))
+                assert torch.equal(mp.validate_edges(p, a, b).cpu(), whole[e0:e0 + c])

@@ -1117,8 +1117,8 @@ def run_ours(args) -> None:
                     "d2h_bytes_per_step": int(d2h)},
             # per step: validate; NEAREST = setup (bucket limits), histogram (+
             # scan), scatter, seeding (+ cuts) and the FP32 filter kernel (+
-            # reduce); NEIGHBORS and path cost one cluster launch each
-            "gpu_launches": 8 * args.steps,
+            # reduce); NEIGHBORS one cluster launch; path cost and its sum
+            "gpu_launches": 9 * args.steps,
             "cpu_baseline": cpu,
             "planner": planner,
             "serving": serving,

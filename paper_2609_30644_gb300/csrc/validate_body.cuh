@@ -1086,7 +1086,9 @@ __device__ __forceinline__ void verdict_body(const VParams &P, float4 *sm4, int 
             int tile = own;
             if (!SHARE) {
                 if (tile >= T || edge_hit) break;
-                if (GROUP && *flag) break;  // another warp's tile collides
+                // another warp's tile collides: one lane reads the flag, which that
+                // warp may be writing, so that the whole warp leaves or stays
+                if (GROUP && __shfl_sync(kFull, lane == 0 ? *flag : 0, 0)) break;
             } else if (T > 1) {
                 if (lane == 0) {
                     tile = T;

@@ -162,15 +162,22 @@ mrpop_status launch_mode(mrpop_problem *p, VParams &V, int warps, size_t smem,
             return MRPOP_OK;
         }
     }
+    if constexpr (MODE == kVerdict && !RA) {
+        const int64_t shared_warps = (int64_t)p->num_sms * bps * warps;
+        if (V.t.L < kShareLinks || V.E > kShareWaves * shared_warps) {
+            // a kernel of its own, with its own shared-memory limit and occupancy
+            kern = p->tuned_regs ? validate_kernel_wide<MODE, RA, false>
+                                 : validate_kernel<MODE, RA, false>;
+            const mrpop_status us = cached_occupancy((const void *)kern, p->device,
+                                                     (int)p->smem_optin, warps * 32, smem, &bps);
+            if (us != MRPOP_OK) return us;
+            if (bps < 1) return set_error(MRPOP_EINVAL, "validation kernel does not fit on an SM");
+        }
+    }
     const int64_t want = (V.E + warps - 1) / warps;
     const int grid = (int)std::min<int64_t>((int64_t)p->num_sms * bps, want);
     V.total_warps = grid * warps;
     V.warps = warps;
-    if constexpr (MODE == kVerdict && !RA) {
-        if (V.t.L < kShareLinks || V.E > kShareWaves * V.total_warps)
-            kern = p->tuned_regs ? validate_kernel_wide<MODE, RA, false>
-                                 : validate_kernel<MODE, RA, false>;
-    }
     kern<<<grid, warps * 32, smem, st>>>(V);
     MRPOP_CUDA_TRY(cudaGetLastError());
     return MRPOP_OK;

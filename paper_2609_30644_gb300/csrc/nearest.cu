@@ -448,11 +448,11 @@ inline mrpop_status scan_rows(const float *tree, int N, int64_t ld, int dim, con
 
 inline mrpop_status nearest_scan(const float *tree, int N, int64_t ld, int dim,
                                  const float *queries, const float *budgets, int Q,
-                                 int64_t *out_idx, cudaStream_t st) {
+                                 int64_t *out_idx, cudaStream_t st, bool no_scratch) {
     int dev = 0, sms = 1, chunk = 0, splits = 1;
     MRPOP_CUDA_TRY(cudaGetDevice(&dev));
     MRPOP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    scan_slices(N, Q, sms, INT64_MAX, &chunk, &splits);
+    scan_slices(N, Q, sms, no_scratch ? (int64_t)kScanCluster * Q : INT64_MAX, &chunk, &splits);
     Best *partial = nullptr;
     const size_t records = (size_t)splits * Q;
     if (splits > kScanCluster)
@@ -2527,6 +2527,7 @@ mrpop_status launch_nearest(const float *tree, int64_t N, int64_t ld, int dim,
                             const float *queries, const float *budgets, int64_t Q,
                             int64_t *out_idx, cudaStream_t st, int filter, int waves) {
     const int n = (int)N, q = (int)Q;
+    bool no_scratch = false;
     // Large batches: budget-ordered tree and queries, expansion filter with
     // exact decisions over shared-memory tree tiles.
     if (takes_sorted(dim, N, Q, filter)) {
@@ -2534,10 +2535,11 @@ mrpop_status launch_nearest(const float *tree, int64_t N, int64_t ld, int dim,
         const mrpop_status s = nearest_sorted_dim(tree, n, ld, dim, queries, budgets, q, out_idx,
                                                   st, nullptr, filter, w);
         // the ordered copies of a tree that nearly fills the device did not
-        // fit: the scan below needs none
+        // fit: the scan needs none, and in one cluster's slices no scratch either
         if (s != MRPOP_ENOMEM) return s;
+        no_scratch = true;
     }
-    return nearest_scan(tree, n, ld, dim, queries, budgets, q, out_idx, st);
+    return nearest_scan(tree, n, ld, dim, queries, budgets, q, out_idx, st, no_scratch);
 }
 
 mrpop_status nearest_pairs(const float *tree, int64_t N, int64_t ld, int dim, const float *queries,

@@ -307,10 +307,10 @@ mrpop_status mrpop_nearest(const float *tree, int64_t n_vertices, int64_t ld, in
                            int64_t *out_idx, void *cuda_stream);
 
 /* Filters of the large-batch NEAREST path (mrpop_nearest_ex).  Large batches
- * (by the product of queries, vertices and dimensions; always from 4,096
- * queries over 2,560 vertices, and from 2,048 queries with the tensor-core
- * filter) order the tree by g and the queries by budget, then pass each
- * (query, vertex) pair through an
+ * (by the product of queries, vertices and dimensions; in dimensions 3, 6, 7,
+ * 14, 21 and 28 also from 4,096 queries over 2,560 vertices, and from 2,048
+ * queries with the tensor-core filter) order the tree by g and the queries by
+ * budget, then pass each (query, vertex) pair through an
  * expansion filter |q|^2 + |x|^2 - 2 q.x <= bound, whose rounding error is
  * bounded so that it never drops the nearest admissible vertex; every vertex
  * that passes is decided with the exact FP32 distance, so the indices do not

@@ -2512,15 +2512,19 @@ static mrpop_status nearest_sorted_dim(const float *tree, int n, int64_t ld, int
 // 16,000 x 8,000 (7.7e8) 120 / 104; 14-D, 64,000 x 2,000 (1.8e9) 174 / 152.
 // With fewer queries a query block's bounds start loose in more slices:
 // 28-D, 64,000 x 1,024 (1.8e9) 158 / 190; 14-D, 256,000 x 1,024 (3.7e9) 305 /
-// 249; 14-D, 1,000,000 x 256 (3.6e9) 298 / 486.  From 4,096 queries over 2,560
-// vertices on, the ordered path is kept below the line too (the scan is up to
-// 25 us faster there), so that batches of that size always skip the pairs
-// whose cost rules them out, as mrpop_nearest_work counts.
+// 249; 14-D, 1,000,000 x 256 (3.6e9) 298 / 486.  In the dimensions of the
+// tensor-core filters alone the ordered path also serves every batch that asks
+// for one, and from 4,096 queries over 2,560 vertices on it is kept below the
+// line, so that batches of that size skip the pairs whose cost rules them out,
+// as mrpop_nearest_work counts (7-D, 3,500 x 4,096: 65 us; the scan is up to 25
+// us faster there).  Elsewhere these two calls would be slower for it: 2,560 x
+// 4,096 in 4-D 31 us by an earlier scan and 60 ordered, in 16-D 45 and 75.
 static bool takes_sorted(int dim, int64_t N, int64_t Q, int filter) {
     if (N <= 0 || !(N <= (1 << 30) || tensor_dim(dim))) return false;
     const double work = (double)N * (double)Q * dim;
     if (Q < 2048) return Q >= 512 && work >= 3e9;
-    return filter == MRPOP_NEAREST_FILTER_TENSOR || work >= 6e8 || (Q >= 4096 && N >= 2560);
+    return work >= 6e8 || (tensor_dim(dim) && (filter == MRPOP_NEAREST_FILTER_TENSOR ||
+                                               (Q >= 4096 && N >= 2560)));
 }
 
 mrpop_status launch_nearest(const float *tree, int64_t N, int64_t ld, int dim,

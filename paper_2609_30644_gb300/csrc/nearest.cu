@@ -2,7 +2,8 @@
 // NEIGHBORS) and path cost (Sec. III-A) over SoA state-cost trees.
 //
 // NEAREST, small batches: an exact scan of every pair in register tiles
-// (nearest_scan_kernel); when the tree is split across blocks (few queries,
+// (nearest_scan_kernel) or, for few pairs, in finer pieces
+// (nearest_small_kernel); when the tree is split across blocks (few queries,
 // large tree), partial bests go to stream-ordered scratch and a second kernel
 // reduces them.  Large batches take the budget-ordered path further down, with
 // an FP32 expansion filter (or, as an option, one on the tensor cores) whose
@@ -344,17 +345,18 @@ nearest_scan_kernel(const float *__restrict__ tree, int N, int64_t ld, int dim,
     cl.sync();  // no block ends while its results are read
 }
 
-// The slices' partial bests of a query, one warp per query.  Launched so that
-// its prologue overlaps the scan's tail; the wait comes before the first read.
+// The slices' partial bests of a query (slice s of query q at q q_step + s s_step),
+// one warp per query.  Launched so that its prologue overlaps the scan's tail;
+// the wait comes before the first read.
 __global__ void __launch_bounds__(256)
-nearest_reduce_kernel(const Best *__restrict__ partial, int splits, int Q,
+nearest_reduce_kernel(const Best *__restrict__ partial, int splits, int Q, int q_step, int s_step,
                       int64_t *__restrict__ out_idx) {
     cudaGridDependencySynchronize();
     const int q = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (q >= Q) return;
     Best b{FLT_MAX * 2.f, FLT_MAX * 2.f, -1};
     for (int s = lane; s < splits; s += 32) {
-        const Best o = partial[(size_t)q * splits + s];
+        const Best o = partial[(size_t)q * q_step + (size_t)s * s_step];
         if (better(o, b)) b = o;
     }
 #pragma unroll
@@ -363,6 +365,22 @@ nearest_reduce_kernel(const Best *__restrict__ partial, int splits, int Q,
         if (better(o, b)) b = o;
     }
     if (lane == 0) out_idx[q] = b.idx;
+}
+
+inline mrpop_status reduce_launch(const Best *partial, int splits, int Q, int q_step, int s_step,
+                                  int64_t *out_idx, cudaStream_t st) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((Q + 7) / 8);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    MRPOP_CUDA_TRY(cudaLaunchKernelEx(&cfg, nearest_reduce_kernel, partial, splits, Q, q_step,
+                                      s_step, out_idx));
+    return MRPOP_OK;
 }
 
 // Slices of the tree for Q queries: two blocks on every SM, whole steps each.
@@ -377,10 +395,10 @@ inline void scan_slices(int N, int Q, int sms, int64_t max_records, int *chunk, 
 }
 
 // The scan of one batch in splits slices.  Up to kScanCluster slices run as
-// one cluster per query tile, which combines its own results: one launch and
-// no scratch (1,000 vertices, 64 queries: 2 us less of host time than a second
-// launch costs).  More write partial, splits records per query, for a second
-// kernel; bounds (or null) is a word per query.
+// one cluster per query tile, which combines its own results: one launch and no
+// scratch (2,000 vertices, 500 queries: 5 us less of host time than a second launch and
+// its scratch cost).  More write partial, splits records per query, for a
+// second kernel; bounds (or null) is a word per query.
 template <int R>
 mrpop_status scan_launch(const float *tree, int N, int64_t ld, int dim, const float *queries,
                          const float *budgets, int Q, int chunk, int splits, int64_t *out_idx,
@@ -413,19 +431,7 @@ mrpop_status scan_launch(const float *tree, int N, int64_t ld, int dim, const fl
     }
     MRPOP_CUDA_TRY(cudaLaunchKernelEx(&cfg, nearest_scan_kernel<R>, tree, N, ld, dim, queries,
                                       budgets, Q, chunk, vec, out_idx, partial, bounds));
-    if (!partial) return MRPOP_OK;
-    at = cudaLaunchAttribute{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg = cudaLaunchConfig_t{};
-    cfg.gridDim = dim3((Q + 7) / 8);
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    MRPOP_CUDA_TRY(cudaLaunchKernelEx(&cfg, nearest_reduce_kernel, (const Best *)partial, splits, Q,
-                                      out_idx));
-    return MRPOP_OK;
+    return partial ? reduce_launch(partial, splits, Q, splits, 1, out_idx, st) : MRPOP_OK;
 }
 
 // Rows per chunk: 6, 7 or 8, whichever pads the dimension least (none for the
@@ -446,14 +452,173 @@ inline mrpop_status scan_rows(const float *tree, int N, int64_t ld, int dim, con
                           bounds, st);
 }
 
+// ---------------------------------------------------------------------------
+// The same scan for few pairs (small_scan), in finer pieces: a block takes 8
+// queries (staged in shared memory) and a slice of at least 1,024 vertices, a
+// thread one vertex at a time against all 8.  Bound by latency: a block of the
+// register tiles above works through 64 queries x 256 vertices at least, alone on
+// its SM while most SMs have none, and its time grows with the dimension (64-D, 500
+// vertices, 500 queries: 27.0 us a call in tiles, 16.4 here, which is the
+// host's; 28-D, 10,000 x 200: 34.2 and 22.6).
+// ---------------------------------------------------------------------------
+constexpr int kSmallThreads = 256;
+constexpr int kSmallQ = 8;
+
+template <int DP>
+__global__ void __launch_bounds__(kSmallThreads)
+nearest_small_kernel(const float *__restrict__ tree, int N, int64_t ld, int dim,
+                     const float *__restrict__ queries, const float *__restrict__ budgets, int Q,
+                     int chunk, int64_t *__restrict__ out_idx, Best *__restrict__ partial) {
+    __shared__ __align__(16) float qs[kSmallQ][DP];
+    __shared__ float cs[kSmallQ];
+    __shared__ Best wbest[kSmallThreads / 32][kSmallQ];
+    const int q0 = blockIdx.x * kSmallQ;
+    const int nq = min(kSmallQ, Q - q0);
+    for (int i = threadIdx.x; i < kSmallQ * DP; i += blockDim.x) {
+        const int j = i / DP, d = i % DP;
+        qs[j][d] = (j < nq && d < dim) ? queries[(size_t)d * Q + q0 + j] : 0.f;
+    }
+    if (threadIdx.x < kSmallQ)
+        cs[threadIdx.x] = threadIdx.x < nq ? budgets[q0 + threadIdx.x] : -FLT_MAX;
+    __syncthreads();
+
+    Best best[kSmallQ];
+#pragma unroll
+    for (int j = 0; j < kSmallQ; ++j) best[j] = Best{FLT_MAX * 2.f, FLT_MAX * 2.f, -1};
+
+    const int vs = blockIdx.y * chunk;
+    const int ve = min(N, vs + chunk);
+    for (int v = vs + threadIdx.x; v < ve; v += blockDim.x) {
+        float x[DP];
+#pragma unroll
+        for (int d = 0; d < DP; ++d) x[d] = d < dim ? __ldg(tree + (size_t)d * ld + v) : 0.f;
+        const float g = __ldg(tree + (size_t)dim * ld + v);
+#pragma unroll
+        for (int j = 0; j < kSmallQ; ++j) {
+            const float4 *q4 = reinterpret_cast<const float4 *>(qs[j]);
+            float d2 = 0.f;
+#pragma unroll
+            for (int d = 0; d < DP / 4; ++d) {
+                const float4 qq = q4[d];
+                const float a0 = qq.x - x[4 * d], a1 = qq.y - x[4 * d + 1];
+                const float a2 = qq.z - x[4 * d + 2], a3 = qq.w - x[4 * d + 3];
+                d2 = fmaf(a0, a0, d2);
+                d2 = fmaf(a1, a1, d2);
+                d2 = fmaf(a2, a2, d2);
+                d2 = fmaf(a3, a3, d2);
+            }
+            if (d2 <= best[j].d2) {
+                // filter of Alg. 2: g_v + |q - q_v| < c (strict)
+                if (g + __fsqrt_rn(d2) < cs[j] && (d2 < best[j].d2 || g < best[j].g)) {
+                    best[j].d2 = d2;
+                    best[j].g = g;
+                    best[j].idx = v;
+                }
+            }
+        }
+    }
+
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int j = 0; j < kSmallQ; ++j) {
+        Best b = best[j];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const Best o = shfl_best(b, off);
+            if (better(o, b)) b = o;
+        }
+        if (lane == 0) wbest[warp][j] = b;
+    }
+    __syncthreads();
+    if (threadIdx.x < nq) {
+        const int j = threadIdx.x;
+        Best b = wbest[0][j];
+        for (int w = 1; w < kSmallThreads / 32; ++w)
+            if (better(wbest[w][j], b)) b = wbest[w][j];
+        if (partial)
+            partial[(size_t)blockIdx.y * Q + q0 + j] = b;
+        else
+            out_idx[q0 + j] = b.idx;
+    }
+}
+
+// Slices of the tree: 8 blocks on every SM, of 1,024 vertices at least.
+inline void small_slices(int N, int Q, int sms, int64_t max_records, int *chunk, int *splits) {
+    const int groups = (Q + kSmallQ - 1) / kSmallQ, target = sms * 8;
+    int s = 1;
+    if (groups < target && N > 4 * kSmallThreads)
+        s = std::min((target + groups - 1) / groups,
+                     (N + 4 * kSmallThreads - 1) / (4 * kSmallThreads));
+    s = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)s, max_records / Q, (int64_t)65535}));
+    const int per = (N + s - 1) / s;
+    *chunk = std::max(1, (per + kSmallThreads - 1) / kSmallThreads) * kSmallThreads;
+    *splits = std::max(1, (N + *chunk - 1) / *chunk);
+}
+
+template <int DP>
+mrpop_status small_launch(const float *tree, int N, int64_t ld, int dim, const float *queries,
+                          const float *budgets, int Q, int chunk, int splits, int64_t *out_idx,
+                          Best *partial, cudaStream_t st) {
+    nearest_small_kernel<DP><<<dim3((Q + kSmallQ - 1) / kSmallQ, splits), kSmallThreads, 0, st>>>(
+        tree, N, ld, dim, queries, budgets, Q, chunk, out_idx, partial);
+    MRPOP_CUDA_TRY(cudaGetLastError());
+    return partial ? reduce_launch(partial, splits, Q, 1, Q, out_idx, st) : MRPOP_OK;
+}
+
+// By the dimension in whole float4s; partial (more than one slice) or null.
+inline mrpop_status small_dims(const float *tree, int N, int64_t ld, int dim, const float *queries,
+                               const float *budgets, int Q, int chunk, int splits,
+                               int64_t *out_idx, Best *partial, cudaStream_t st) {
+#define MRPOP_SMALL_DIM(D)                                                                    \
+    if (dim <= D)                                                                             \
+        return small_launch<D>(tree, N, ld, dim, queries, budgets, Q, chunk, splits, out_idx, \
+                               partial, st)
+    MRPOP_SMALL_DIM(4);
+    MRPOP_SMALL_DIM(8);
+    MRPOP_SMALL_DIM(12);
+    MRPOP_SMALL_DIM(16);
+    MRPOP_SMALL_DIM(20);
+    MRPOP_SMALL_DIM(24);
+    MRPOP_SMALL_DIM(28);
+    MRPOP_SMALL_DIM(32);
+    MRPOP_SMALL_DIM(48);
+    MRPOP_SMALL_DIM(64);
+#undef MRPOP_SMALL_DIM
+    return set_error(MRPOP_EINVAL, "nearest: dimension %d", dim);
+}
+
+// Whether a scan of N vertices for Q queries takes the finer pieces, by pairs and
+// by what either form launches.  Up to 1,024 vertices both are one launch (tiles /
+// pieces, us: 28-D, 1,000 x 1,000 20.7 / 17.4; 45-D 24.7 / 20.7; 28-D, 500 x
+// 5,000 26.9 / 23.0), but pieces of more than 32 dimensions have rows for 48 or 64
+// (35-D, 1,000 x 2,000 22.5 / 24.8).  Up to 2,048 the tiles are one cluster launch
+// and the pieces two kernels and their scratch (14-D, 2,000 x 500 16.5 / 22.1; 28-D
+// 20.9 / 22.3; 45-D 25.1 / 23.5).  Above, both are two kernels (28-D, 10,000 x 200
+// 34.2 / 22.6; 45-D, 30,000 x 64 32.0 / 27.2; 28-D, 4,000 x 1,000 30.7 / 33.3).
+inline bool small_scan(int dim, int N, int Q) {
+    const int64_t pairs = (int64_t)N * Q;
+    if (N <= 4 * kSmallThreads) return pairs <= (dim > 32 ? 1500000 : 3500000);
+    if (N <= kScanCluster * kScanV) return dim > 32 && pairs <= 2000000;
+    return pairs <= 2500000;
+}
+
 inline mrpop_status nearest_scan(const float *tree, int N, int64_t ld, int dim,
                                  const float *queries, const float *budgets, int Q,
                                  int64_t *out_idx, cudaStream_t st, bool no_scratch) {
     int dev = 0, sms = 1, chunk = 0, splits = 1;
     MRPOP_CUDA_TRY(cudaGetDevice(&dev));
     MRPOP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    scan_slices(N, Q, sms, no_scratch ? (int64_t)kScanCluster * Q : INT64_MAX, &chunk, &splits);
     Best *partial = nullptr;
+    if (!no_scratch && small_scan(dim, N, Q)) {
+        small_slices(N, Q, sms, INT64_MAX, &chunk, &splits);
+        if (splits > 1)
+            MRPOP_CUDA_TRY(scratch_alloc((void **)&partial, sizeof(Best) * (size_t)splits * Q, st));
+        const mrpop_status s = small_dims(tree, N, ld, dim, queries, budgets, Q, chunk, splits,
+                                          out_idx, partial, st);
+        if (partial) cudaFreeAsync(partial, st);
+        return s;
+    }
+    scan_slices(N, Q, sms, no_scratch ? (int64_t)kScanCluster * Q : INT64_MAX, &chunk, &splits);
     const size_t records = (size_t)splits * Q;
     if (splits > kScanCluster)
         MRPOP_CUDA_TRY(scratch_alloc((void **)&partial,
@@ -2727,6 +2892,11 @@ extern "C" mrpop_status mrpop_nearest_noalloc(const float *tree, int64_t N, int6
     int dev = 0, sms = 1, chunk = 0, splits = 1;
     MRPOP_CUDA_TRY(cudaGetDevice(&dev));
     MRPOP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (small_scan(dim, n, q)) {
+        small_slices(n, q, sms, kNoAllocRecords, &chunk, &splits);
+        return small_dims(tree, n, ld, dim, queries, budgets, q, chunk, splits, out_idx,
+                          splits > 1 ? scratch : nullptr, st);
+    }
     scan_slices(n, q, sms, kNoAllocRecords, &chunk, &splits);
     return scan_rows(tree, n, ld, dim, queries, budgets, q, chunk, splits, out_idx,
                      splits > kScanCluster ? scratch : nullptr, nullptr, st);

@@ -85,3 +85,52 @@ def test_small_work_takes_the_scan(mp, D, n, Q):
                       for i in range(0, Q, 64)])
     for filt in (0, 1):
         assert torch.equal(mp.nearest(tree, q, c, filter=filt), want)
+
+
+def _scan_against_oracle(mp, orc, D, n, Q):
+    if n > 4:
+        lo, hi = -2.9 * np.ones(D), 2.9 * np.ones(D)
+        diag = float(np.sqrt(D) * 5.8)
+        tree = synth.random_tree_fast(D, n + 5, lo, hi, seed=D + n)
+        qs, cs = synth.nn_queries(D, Q, lo, hi, seed=D + n + 1, budget_lo=0.3 * diag,
+                                  budget_hi=1.9 * diag)
+        k = min(n // 4, 40)                   # exact ties, some with equal g
+        tree[:, n - k:n] = tree[:, :k]
+        tree[D, n - k:n - k // 2] += np.float32(0.5)
+        qs[:, :min(k, Q)] = tree[:D, :min(k, Q)]
+    else:
+        tree = np.zeros((D + 1, 6), np.float32)
+        qs, cs = np.ones((D, Q), np.float32), np.full(Q, 9.0, np.float32)
+    t, q, c = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (tree, qs, cs))
+    got = mp.nearest(t, q, c, n_vertices=n).cpu().numpy()
+    noalloc = torch.full((Q,), -7, dtype=torch.int64, device="cuda")
+    assert mp.lib.mrpop_nearest_noalloc(t.data_ptr(), n, tree.shape[1], D, q.data_ptr(),
+                                        c.data_ptr(), Q, noalloc.data_ptr(),
+                                        torch.cuda.current_stream().cuda_stream) == 0
+    np.testing.assert_array_equal(noalloc.cpu().numpy(), got)
+    for i in range(0, Q, max(1, Q // 60)):
+        ref, bd, sd, gap = orc.nearest(tree, qs[:, i], cs[i], n_vertices=n)
+        # a different vertex only where FP32 cannot tell the two apart
+        assert got[i] == ref or (np.isfinite(sd) and sd - bd <= 1e-5 * max(bd, 1e-30)) or \
+            gap <= 1e-5 * max(1.0, abs(float(cs[i]))), (i, got[i], ref)
+
+
+# few pairs, in pieces of 8 queries: every padded dimension at and above its
+# rows, one slice and several, ragged slices and query groups
+@pytest.mark.parametrize("D", [1, 4, 5, 8, 9, 12, 13, 16, 17, 20, 21, 24, 25, 28, 29, 32, 33, 48, 49,
+                               64])
+@pytest.mark.parametrize("n,Q", [(1, 1), (255, 9), (1024, 64), (2049, 33), (5003, 257), (40001, 7)])
+def test_scan_of_few_pairs(mp, orc, D, n, Q):
+    _scan_against_oracle(mp, orc, D, n, Q)
+
+
+# the register tiles above that: one slice, clusters of slices, slices with a
+# second kernel; rows of 6, 7 and 8 with and without padding; both sides of the
+# lines between the two forms
+@pytest.mark.parametrize("D,n,Q", [(7, 1025, 64), (8, 1500, 65), (9, 2047, 63), (32, 2048, 2),
+                                   (33, 2048, 976), (33, 2048, 977), (13, 2049, 1220),
+                                   (13, 2049, 1221), (28, 5003, 600), (35, 20001, 140), (64, 3001, 900),
+                                   (3, 1000, 3500), (3, 1000, 3501), (6, 300, 12001), (64, 999, 1600),
+                                   (35, 1000, 1500), (35, 1000, 1501)])
+def test_scan_in_tiles(mp, orc, D, n, Q):
+    _scan_against_oracle(mp, orc, D, n, Q)

@@ -395,9 +395,10 @@ inline void scan_slices(int N, int Q, int sms, int64_t max_records, int *chunk, 
 }
 
 // The scan of one batch in splits slices.  Up to kScanCluster slices run as
-// one cluster per query tile, which combines its own results: one launch and no
-// scratch (2,000 vertices, 500 queries: 5 us less of host time than a second launch and
-// its scratch cost).  More write partial, splits records per query, for a
+// one cluster per query tile where the chip holds all clusters at once
+// (scan_in_clusters), which combines its own results: one launch and no scratch
+// (2,000 vertices, 500 queries: 5 us less of host time than a second launch and
+// its scratch cost).  Others write partial, splits records per query, for a
 // second kernel; bounds (or null) is a word per query.
 template <int R>
 mrpop_status scan_launch(const float *tree, int N, int64_t ld, int dim, const float *queries,
@@ -602,6 +603,41 @@ inline bool small_scan(int dim, int N, int Q) {
     return pairs <= 2500000;
 }
 
+// Whether the scan's slices run as clusters of one query tile each.  The blocks of
+// a cluster share a GPC, so a chip of two blocks on each of 152 SMs holds 36
+// clusters of 8 at once, 38 of 7, 46 of 6, 58 of 5, 74 of 4, 97 of 3; one more
+// is a second wave (14-D, 12,188 vertices in 6 slices, 3,000 queries, 47 clusters:
+// 91.1 us, with scratch 63.2; 8,092 in 4, 4,500 queries, 71 clusters: 64.1 and 64.4).
+inline mrpop_status scan_in_clusters(int splits, int Q, bool *out) {
+    static std::atomic<int> active[64][kScanCluster + 1];  // of the device; 0: not asked yet
+    *out = splits <= kScanCluster;
+    if (!*out || splits <= 1) return MRPOP_OK;
+    int dev = 0;
+    MRPOP_CUDA_TRY(cudaGetDevice(&dev));
+    int n = dev < 64 ? active[dev][splits].load() : 0;
+    if (n == 0) {
+        // the largest tables, of which two blocks still fit an SM
+        const size_t smem = scan_smem_bytes(MRPOP_MAX_LINKS, 8);
+        MRPOP_CUDA_TRY(cudaFuncSetAttribute(nearest_scan_kernel<8>,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = 1;
+        at.val.clusterDim.y = splits;
+        at.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(1, splits);
+        cfg.blockDim = dim3(kScanThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        MRPOP_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, nearest_scan_kernel<8>, &cfg));
+        if (dev < 64) active[dev][splits].store(n);
+    }
+    *out = (Q + kScanQ - 1) / kScanQ <= n;
+    return MRPOP_OK;
+}
+
 inline mrpop_status nearest_scan(const float *tree, int N, int64_t ld, int dim,
                                  const float *queries, const float *budgets, int Q,
                                  int64_t *out_idx, cudaStream_t st, bool no_scratch) {
@@ -620,7 +656,12 @@ inline mrpop_status nearest_scan(const float *tree, int N, int64_t ld, int dim,
     }
     scan_slices(N, Q, sms, no_scratch ? (int64_t)kScanCluster * Q : INT64_MAX, &chunk, &splits);
     const size_t records = (size_t)splits * Q;
-    if (splits > kScanCluster)
+    bool clusters = true;
+    if (!no_scratch) {
+        const mrpop_status s = scan_in_clusters(splits, Q, &clusters);
+        if (s != MRPOP_OK) return s;
+    }
+    if (!clusters)
         MRPOP_CUDA_TRY(scratch_alloc((void **)&partial,
                                      sizeof(Best) * records + sizeof(unsigned) * (size_t)Q, st));
     const mrpop_status s =
@@ -2898,6 +2939,8 @@ extern "C" mrpop_status mrpop_nearest_noalloc(const float *tree, int64_t N, int6
                           splits > 1 ? scratch : nullptr, st);
     }
     scan_slices(n, q, sms, kNoAllocRecords, &chunk, &splits);
+    bool clusters = true;
+    if ((s = scan_in_clusters(splits, q, &clusters)) != MRPOP_OK) return s;
     return scan_rows(tree, n, ld, dim, queries, budgets, q, chunk, splits, out_idx,
-                     splits > kScanCluster ? scratch : nullptr, nullptr, st);
+                     clusters ? nullptr : scratch, nullptr, st);
 }

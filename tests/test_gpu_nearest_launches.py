@@ -131,6 +131,9 @@ def test_scan_of_few_pairs(mp, orc, D, n, Q):
                                    (33, 2048, 976), (33, 2048, 977), (13, 2049, 1220),
                                    (13, 2049, 1221), (28, 5003, 600), (35, 20001, 140), (64, 3001, 900),
                                    (3, 1000, 3500), (3, 1000, 3501), (6, 300, 12001), (64, 999, 1600),
-                                   (35, 1000, 1500), (35, 1000, 1501)])
+                                   (35, 1000, 1500), (35, 1000, 1501),
+                                   # clusters that fill the chip, one more and their scratch
+                                   (8, 4000, 2304), (8, 4000, 2305), (14, 3000, 2944), (14, 3000, 2945),
+                                   (6, 2000, 4736), (6, 2000, 4737), (4, 2000, 9729)])
 def test_scan_in_tiles(mp, orc, D, n, Q):
     _scan_against_oracle(mp, orc, D, n, Q)

@@ -2782,8 +2782,10 @@ mrpop_status launch_neighbors(const float *tree, int64_t N, int64_t ld, int dim,
     const int ranges = (int)std::min<int64_t>(std::min<int64_t>(want, (N + kNbTile - 1) / kNbTile),
                                               std::max<int64_t>(1, 65535));
     // short lists in up to 16 dimensions: the ranges as one cluster, up to
-    // 65,536 vertices (8,192 a block; beyond, more ranges repay the merge)
-    if (k_max <= kNbListMax && dim <= 16 && N <= 65536 && Q > 0) {
+    // 65,536 vertices (8,192 a block; beyond, more ranges repay the merge), for a
+    // single query up to 24,576 above 4 dimensions (its 8 blocks leave the chip
+    // idle: 7-D, 48,000 vertices 46.0 us, in ranges 31.9; 24,000 25.8 and 26.4)
+    if (k_max <= kNbListMax && dim <= 16 && N <= (Q == 1 && dim > 4 ? 24576 : 65536) && Q > 0) {
         const int r = std::max(1, std::min(ranges, kNbCluster)), n = (int)N, q = (int)Q,
                   k = (int)k_max;
         if (dim <= 4)

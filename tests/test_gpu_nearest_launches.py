@@ -137,3 +137,26 @@ def test_scan_of_few_pairs(mp, orc, D, n, Q):
                                    (6, 2000, 4736), (6, 2000, 4737), (4, 2000, 9729)])
 def test_scan_in_tiles(mp, orc, D, n, Q):
     _scan_against_oracle(mp, orc, D, n, Q)
+
+
+# one query on either side of its line to the ranges, and two
+@pytest.mark.parametrize("D,n,Q", [(7, 24576, 1), (7, 24577, 1), (16, 40001, 1), (4, 40001, 1),
+                                   (7, 40001, 2)])
+@pytest.mark.parametrize("k_max", [8, 64])
+def test_neighbors_of_few_queries(mp, orc, D, n, Q, k_max):
+    rng = np.random.default_rng(D * n)
+    tree = np.zeros((D + 1, n), np.float32)   # the last row is g, which is not read
+    tree[:D] = rng.uniform(-2.9, 2.9, (D, n))
+    qs = rng.uniform(-1.0, 1.0, (D, Q)).astype(np.float32)
+    delta = np.float32({4: 0.7, 7: 1.8, 16: 5.0}[D])
+    idx, cnt = mp.neighbors(torch.from_numpy(tree).cuda(), torch.from_numpy(qs).cuda(),
+                            float(delta), k_max, dim=D)
+    idx, cnt = idx.cpu().numpy(), cnt.cpu().numpy()
+    for i in range(Q):
+        ref, rc, gap = orc.neighbors(tree, qs[:, i], delta, k_max)
+        if gap <= 1e-5 * delta:               # FP32 cannot decide a vertex
+            assert abs(int(cnt[i]) - rc) <= 2
+            continue
+        assert cnt[i] == rc and rc > 0
+        np.testing.assert_array_equal(idx[i, :min(rc, k_max)], ref[:k_max])
+        assert (idx[i, min(rc, k_max):] == -1).all()

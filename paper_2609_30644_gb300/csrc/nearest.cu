@@ -2535,8 +2535,10 @@ constexpr int kPathThreads = 512;
 // blocks' sums in block order: one launch and no scratch (16,385 vertices in
 // 14-D: 12.3 us with a cold L2, 17.5 with 4-byte loads and a second kernel).
 // Longer paths need more SMs to read from memory (65,537 vertices in 14-D, cold:
-// 28.7 us as a cluster, 13.3 as 64 blocks; 131,073: 47 and 15.4): their blocks
-// write their sums to partial, which a second kernel adds.
+// 28.7 us as a cluster, 13.3 as 64 blocks; 131,073: 47 and 15.4), and so do
+// 4-byte loads above 350,000 floats (35-D, 8,001 vertices 16.4 us a call as a
+// cluster and 21.0 in blocks, 10,001 19.4 and 19.4, 16,001 27.2 and 19.9): their
+// blocks write their sums to partial, which a second kernel adds.
 template <int V>
 __global__ void __launch_bounds__(kPathThreads)
 path_cost_kernel(const float *__restrict__ path, int64_t M, int dim, int64_t chunk,
@@ -2823,7 +2825,7 @@ static mrpop_status path_cost_v(const float *path, int64_t M, int dim, double *o
                                 cudaStream_t st) {
     const int64_t segs = M > 1 ? M - 1 : 0;
     constexpr int64_t kBlockSegs = 2 * kPathThreads;
-    if (segs <= 16384) {
+    if (segs <= 16384 && (V > 1 || segs * dim <= 350000)) {
         int blocks = 1;
         while (blocks < 8 && blocks * kBlockSegs < segs) blocks *= 2;
         cudaLaunchAttribute at{};

@@ -160,3 +160,15 @@ def test_neighbors_of_few_queries(mp, orc, D, n, Q, k_max):
         assert cnt[i] == rc and rc > 0
         np.testing.assert_array_equal(idx[i, :min(rc, k_max)], ref[:k_max])
         assert (idx[i, min(rc, k_max):] == -1).all()
+
+
+# odd dimensions (4-byte loads) on both sides of 350,000 floats in a path
+@pytest.mark.parametrize("D,M", [(35, 10001), (35, 10002), (63, 5556), (63, 5557), (35, 16385),
+                                 (23, 15218), (23, 15219)])
+def test_path_cost_of_odd_dimensions(mp, D, M):
+    p = torch.from_numpy(np.random.default_rng(M).uniform(-2.9, 2.9, (M, D)).astype(np.float32)).cuda()
+    got = mp.path_cost(p).item()
+    ref = (p[1:].double() - p[:-1].double()).norm(dim=1).sum().item()
+    # FP32 segment lengths: (D + 3) roundings of 2^-24 each at most
+    assert abs(got - ref) <= (D + 3) * 2.0 ** -24 * ref
+    assert mp.path_cost(p).item() == got

@@ -1427,7 +1427,8 @@ struct F32Shape {
     // the tile's registers do not spill (they do below 8 dimensions)
     static constexpr bool PACKED = DIM >= 8 && DIM <= 21;
     // vertices per shared-memory tile (six 64-vertex steps per barrier up to
-    // 14 dimensions) such that two blocks of 256 threads fit an SM
+    // 14 dimensions) such that two blocks of 256 threads fit an SM up to 56
+    // rows (64 rows: 121 KB a block, one per SM)
     static constexpr int VT = DIM <= 14 ? 384 : (DIM <= 21 && !PACKED) ? 128 : 64;
     static constexpr int ROWS = DIM + 2;              // x_d, g, folded |x|^2
     static constexpr int AM = PACKED ? 2 : 1;         // copies of each -2 q_d
@@ -2368,11 +2369,11 @@ neighbors_kernel(const float *__restrict__ tree, int N, int64_t ld, int dim,
 // Each warp scans its range for its query, the query in registers and the
 // distance compared squared (thr: the largest float whose square root is
 // within delta), and keeps its list in shared memory; then the blocks read one
-// another's counts and write their part of each list in place.  Writing the
-// ranges' lists to scratch and concatenating them in a second kernel, one
-// thread per query, took 22 + 10 us for 1,024 queries over 4,096 vertices in
-// 7-D and an allocation (28.9 us a call); a call takes 20.6 us now, most of that
-// the host's.
+// another's counts and write their part of each list in place.  1,024 queries
+// over 4,096 vertices in 7-D: 14.5 us (ncu, cold L2); writing the ranges' lists to
+// scratch and concatenating them in a second kernel, one thread per query, 20.2 +
+// 7.9 and an allocation.  A call, which the host bounds, 20.9 to 26.7 us over four
+// runs, 28.8 to 29.4 that way.
 constexpr int kNbListMax = 64;
 constexpr int kNbCluster = 8;
 

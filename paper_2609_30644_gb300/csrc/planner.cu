@@ -456,10 +456,9 @@ __global__ void k_solution(const Slot *__restrict__ slots) {
 }
 
 // Path of the winning iteration: root_a .. z_new, then z_conn .. root_b.
-// One thread follows the parents; the configurations are written to
-// out_q [cap][D] in that order (reversed to start -> goal by the host when the
+// One thread follows the parents; the block then copies the configurations to
+// out_q [cap][D] in that order (reversed to start -> goal by the caller when the
 // expanded tree was the goal tree).
-// One thread follows the parents; the block then copies the configurations.
 __device__ __forceinline__ void extract_body(const Slot &S, int it, int *scratch, float *out_q,
                                              int cap, int *len_out) {
     __shared__ int s_na, s_n;
@@ -1786,10 +1785,11 @@ static mrpop_status plan_batch(mrpop_problem *const *ps, int n, double budget, i
 // all of the problem's robots at once (their roadmaps and random streams are
 // independent, and a round is a chain of short phases, K times as long robot
 // by robot: twelve problems of 2-8 arms, 24 steps, 77 ms of kernel time robot
-// by robot and 62 ms with the phases over all robots and link_body); a search step is the nine phases of the stepped form; an
-// incumbent candidate is re-checked at a quarter of the resolution -- and
-// each phase is cut into chunks (256 samples or iterations, 16 NEAREST
-// queries, 32 edges, 8 NEIGHBORS queries).  CTAs claim chunks of any problem
+// by robot and 62 ms with the phases over all robots and link_body); a search
+// step is the nine phases of the stepped form; an incumbent candidate is
+// re-checked at a quarter of the resolution -- and each phase is cut into
+// chunks (256 roadmap samples, 16 search samples, 16 NEAREST queries, 8 roadmap
+// candidates, up to 32 edges, 8 NEIGHBORS queries).  CTAs claim chunks of any problem
 // with one atomic add on the problem's phase word, which carries the phase
 // itself (kind, chunk count) beside the next chunk, so a claim always
 // names the phase it belongs to.  The CTA that finishes a phase's last chunk

@@ -149,7 +149,7 @@ mrpop_status launch_mode(mrpop_problem *p, VParams &V, int warps, size_t smem,
                                              warps * 32, smem, &bps);
     if (os != MRPOP_OK) return os;
     if (bps < 1) return set_error(MRPOP_EINVAL, "validation kernel does not fit on an SM");
-    // few edges: 256 planar edges took 18.6 us with an edge per warp, 13.4 us here
+    // few edges: 256 planar edges 12.3 us (ncu, cold L2), 18.0 with an edge per warp
     if (MODE == kVerdict && !RA && warps > 1 && V.E <= kGroupWaves * p->num_sms * bps) {
         int gbps = 0;
         const mrpop_status gs = cached_occupancy((const void *)validate_group_kernel, p->device,
@@ -197,8 +197,9 @@ mrpop_status launch_spl(mrpop_problem *p, VParams &V, int warps, size_t smem,
 // configuration and robot (blockIdx.y), the robot's table rows in shared
 // memory.  Bound by the stores of the sphere centres, 12 bytes a sphere: read
 // from global memory link by link and sphere by sphere, the table's latency
-// was most of the time (20,001 configurations of two 60-sphere arms, 29 MB,
-// which need 4.4 us: a call 21.0 us, now 15.7, most of that the host's).
+// was most of the time (20,001 configurations of two 60-sphere arms, 29 MB, which
+// need 4.4 us: 24.7 us so, 9.8 here (ncu, cold L2); a call 22.5 and 15.8 to 18.5,
+// the host's).
 // ---------------------------------------------------------------------------
 constexpr int kFkThreads = 128;
 

@@ -107,13 +107,18 @@ static cudaError_t scratch_pool(cudaMemPool_t *out) {
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
         cudaMemPool_t pool = nullptr;
-        if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
-        unsigned long long keep = 1ull << 30;
-        if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) !=
-            cudaSuccess) {
-            cudaMemPoolDestroy(pool);
-            return e;
+        // the first call that needs scratch may be one that is being captured,
+        // which a pool made in the capture's own mode would invalidate
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        e = cudaMemPoolCreate(&pool, &props);
+        if (e == cudaSuccess) {
+            unsigned long long keep = 1ull << 30;
+            e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) cudaMemPoolDestroy(pool);
         }
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) return e;
         g_pool[dev] = pool;
     }
     *out = g_pool[dev];

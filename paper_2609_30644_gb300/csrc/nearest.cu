@@ -254,7 +254,7 @@ nearest_scan_kernel(const float *__restrict__ tree, int N, int64_t ld, int dim,
             rows |= m <= lim[r] ? 1u << r : 0u;
         }
         const unsigned any = __reduce_or_sync(kFull, rows);
-        const int v0 = vs + s * kScanV;
+        const int v0 = vs + s * kScanV, nv = min(kScanV, ve - v0);
         const float *gs = gt + (s & 3) * kScanV;
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
@@ -265,6 +265,10 @@ nearest_scan_kernel(const float *__restrict__ tree, int N, int64_t ld, int dim,
                 d2[2 * p] = f32x2_lo(acc2[r][p]);
                 d2[2 * p + 1] = f32x2_hi(acc2[r][p]);
             }
+            if (nv < kScanV)  // columns past the slice are zeros, which may lie near a query
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (4 * lane + (k < 4 ? k : 124 + k) >= nv) d2[k] = FLT_MAX * 2.f;
             const float c = cq[warp * 8 + r];
             float bd = sb_d2[r][tid], lr = lim[r];
             int bv = sb_v[r][tid];

@@ -458,13 +458,13 @@ inline mrpop_status scan_rows(const float *tree, int N, int64_t ld, int dim, con
 }
 
 // ---------------------------------------------------------------------------
-// The same scan for few pairs (small_scan), in finer pieces: a block takes 8
-// queries (staged in shared memory) and a slice of at least 1,024 vertices, a
-// thread one vertex at a time against all 8.  Bound by latency: a block of the
-// register tiles above works through 64 queries x 256 vertices at least, alone on
-// its SM while most SMs have none, and its time grows with the dimension (64-D, 500
-// vertices, 500 queries: 27.0 us a call in tiles, 16.4 here, which is the
-// host's; 28-D, 10,000 x 200: 34.2 and 22.6).
+// The same scan for few pairs in more than 16 dimensions (small_scan), in finer
+// pieces: a block takes 8 queries (staged in shared memory) and a slice of at
+// least 1,024 vertices, a thread one vertex at a time against all 8.  Bound by
+// latency: a block of the register tiles above works through 64 queries x 256
+// vertices at least, alone on its SM while most SMs have none, and its time grows
+// with the dimension (64-D, 450 vertices, 1,200 queries: 24.9 us a call in tiles,
+// 16.9 here, which is the host's; 28-D, 2,100 x 1,200: 29.0 and 22.0).
 // ---------------------------------------------------------------------------
 constexpr int kSmallThreads = 256;
 constexpr int kSmallQ = 8;
@@ -549,15 +549,15 @@ nearest_small_kernel(const float *__restrict__ tree, int N, int64_t ld, int dim,
 
 // Slices of the tree: 8 blocks on every SM, of 1,024 vertices at least.
 inline void small_slices(int N, int Q, int sms, int64_t max_records, int *chunk, int *splits) {
-    const int groups = (Q + kSmallQ - 1) / kSmallQ, target = sms * 8;
-    int s = 1;
-    if (groups < target && N > 4 * kSmallThreads)
-        s = std::min((target + groups - 1) / groups,
-                     (N + 4 * kSmallThreads - 1) / (4 * kSmallThreads));
-    s = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)s, max_records / Q, (int64_t)65535}));
-    const int per = (N + s - 1) / s;
-    *chunk = std::max(1, (per + kSmallThreads - 1) / kSmallThreads) * kSmallThreads;
-    *splits = std::max(1, (N + *chunk - 1) / *chunk);
+    const int64_t n = N, groups = ((int64_t)Q + kSmallQ - 1) / kSmallQ, target = (int64_t)sms * 8;
+    int64_t s = 1;
+    if (groups < target && n > 4 * kSmallThreads)
+        s = std::min((target + groups - 1) / groups, (n + 4 * kSmallThreads - 1) / (4 * kSmallThreads));
+    s = std::max<int64_t>(1, std::min<int64_t>({s, max_records / Q, 65535}));
+    const int64_t c = std::max<int64_t>(
+        kSmallThreads, ((n + s - 1) / s + kSmallThreads - 1) / kSmallThreads * kSmallThreads);
+    *chunk = (int)std::min<int64_t>(c, (int64_t)1 << 30);
+    *splits = (int)std::max<int64_t>(1, (n + *chunk - 1) / *chunk);
 }
 
 template <int DP>
@@ -578,10 +578,6 @@ inline mrpop_status small_dims(const float *tree, int N, int64_t ld, int dim, co
     if (dim <= D)                                                                             \
         return small_launch<D>(tree, N, ld, dim, queries, budgets, Q, chunk, splits, out_idx, \
                                partial, st)
-    MRPOP_SMALL_DIM(4);
-    MRPOP_SMALL_DIM(8);
-    MRPOP_SMALL_DIM(12);
-    MRPOP_SMALL_DIM(16);
     MRPOP_SMALL_DIM(20);
     MRPOP_SMALL_DIM(24);
     MRPOP_SMALL_DIM(28);
@@ -592,19 +588,21 @@ inline mrpop_status small_dims(const float *tree, int N, int64_t ld, int dim, co
     return set_error(MRPOP_EINVAL, "nearest: dimension %d", dim);
 }
 
-// Whether a scan of N vertices for Q queries takes the finer pieces, by pairs and
-// by what either form launches.  Up to 1,024 vertices both are one launch (tiles /
-// pieces, us: 28-D, 1,000 x 1,000 20.7 / 17.4; 45-D 24.7 / 20.7; 28-D, 500 x
-// 5,000 26.9 / 23.0), but pieces of more than 32 dimensions have rows for 48 or 64
-// (35-D, 1,000 x 2,000 22.5 / 24.8).  Up to 2,048 the tiles are one cluster launch
-// and the pieces two kernels and their scratch (14-D, 2,000 x 500 16.5 / 22.1; 28-D
-// 20.9 / 22.3; 45-D 25.1 / 23.5).  Above, both are two kernels (28-D, 10,000 x 200
-// 34.2 / 22.6; 45-D, 30,000 x 64 32.0 / 27.2; 28-D, 4,000 x 1,000 30.7 / 33.3).
-inline bool small_scan(int dim, int N, int Q) {
-    const int64_t pairs = (int64_t)N * Q;
-    if (N <= 4 * kSmallThreads) return pairs <= (dim > 32 ? 1500000 : 3500000);
-    if (N <= kScanCluster * kScanV) return dim > 32 && pairs <= 2000000;
-    return pairs <= 2500000;
+// Whether a scan of N vertices for Q queries takes the finer pieces: where their
+// blocks are one wave (two per SM fit of more than 32 dimensions, three below).
+// Tiles / pieces (us): up to 1,024 vertices, one launch of either, 64-D 450 x 2,400
+// 24.9 / 17.7, 450 x 4,000 25.1 / 31.1, 28-D 1,024 x 2,400 22.8 / 18.2, x 4,000 23.1 /
+// 31.1.  Up to 2,048 the tiles are one cluster launch and the pieces two kernels
+// and their scratch (28-D, 1,500 x 700 18.2 / 23.0; 64-D 24.0 / 25.2).  Above, both
+// are two kernels (28-D, 10,000 x 300 25.8 / 25.2, 3,000 x 1,200 29.1 / 25.2; 64-D,
+// 10,000 x 64 27.6 / 23.4, but beyond a block per SM 5,000 x 300 26.7 / 29.4).  Up to
+// 16 dimensions the tiles are bound by the host's call there.
+inline bool small_scan(int dim, int N, int Q, int sms, int64_t max_records) {
+    if (dim <= 16 || (N > 4 * kSmallThreads && N <= kScanCluster * kScanV)) return false;
+    int chunk = 0, splits = 1;
+    small_slices(N, Q, sms, max_records, &chunk, &splits);
+    const int per_sm = N <= 4 * kSmallThreads ? 2 : dim <= 32 ? 3 : 1;
+    return ((int64_t)Q + kSmallQ - 1) / kSmallQ * splits <= (int64_t)per_sm * sms;
 }
 
 // Whether the scan's slices run as clusters of one query tile each.  The blocks of
@@ -649,7 +647,7 @@ inline mrpop_status nearest_scan(const float *tree, int N, int64_t ld, int dim,
     MRPOP_CUDA_TRY(cudaGetDevice(&dev));
     MRPOP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     Best *partial = nullptr;
-    if (!no_scratch && small_scan(dim, N, Q)) {
+    if (!no_scratch && small_scan(dim, N, Q, sms, INT64_MAX)) {
         small_slices(N, Q, sms, INT64_MAX, &chunk, &splits);
         if (splits > 1)
             MRPOP_CUDA_TRY(scratch_alloc((void **)&partial, sizeof(Best) * (size_t)splits * Q, st));
@@ -2942,7 +2940,7 @@ extern "C" mrpop_status mrpop_nearest_noalloc(const float *tree, int64_t N, int6
     int dev = 0, sms = 1, chunk = 0, splits = 1;
     MRPOP_CUDA_TRY(cudaGetDevice(&dev));
     MRPOP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (small_scan(dim, n, q)) {
+    if (small_scan(dim, n, q, sms, kNoAllocRecords)) {
         small_slices(n, q, sms, kNoAllocRecords, &chunk, &splits);
         return small_dims(tree, n, ld, dim, queries, budgets, q, chunk, splits, out_idx,
                           splits > 1 ? scratch : nullptr, st);

@@ -115,23 +115,23 @@ def _scan_against_oracle(mp, orc, D, n, Q):
             gap <= 1e-5 * max(1.0, abs(float(cs[i]))), (i, got[i], ref)
 
 
-# few pairs, in pieces of 8 queries: every padded dimension at and above its
-# rows, one slice and several, ragged slices and query groups
-@pytest.mark.parametrize("D", [1, 4, 5, 8, 9, 12, 13, 16, 17, 20, 21, 24, 25, 28, 29, 32, 33, 48, 49,
-                               64])
+# few pairs, in pieces of 8 queries above 16 dimensions: every padded dimension at
+# and above its rows, one slice and several, ragged slices and query groups
+@pytest.mark.parametrize("D", [1, 4, 5, 8, 13, 16, 17, 20, 21, 24, 25, 28, 29, 32, 33, 48, 49, 64])
 @pytest.mark.parametrize("n,Q", [(1, 1), (255, 9), (1024, 64), (2049, 33), (5003, 257), (40001, 7)])
 def test_scan_of_few_pairs(mp, orc, D, n, Q):
     _scan_against_oracle(mp, orc, D, n, Q)
 
 
-# the register tiles above that: one slice, clusters of slices, slices with a
-# second kernel; rows of 6, 7 and 8 with and without padding; both sides of the
-# lines between the two forms
+# the register tiles: one slice, clusters of slices, slices with a second kernel;
+# rows of 6, 7 and 8 with and without padding; last steps of one and of all but one
+# vertex; both sides of the lines between the two forms
 @pytest.mark.parametrize("D,n,Q", [(7, 1025, 64), (8, 1500, 65), (9, 2047, 63), (32, 2048, 2),
-                                   (33, 2048, 976), (33, 2048, 977), (13, 2049, 1220),
-                                   (13, 2049, 1221), (28, 5003, 600), (35, 20001, 140), (64, 3001, 900),
-                                   (3, 1000, 3500), (3, 1000, 3501), (6, 300, 12001), (64, 999, 1600),
-                                   (35, 1000, 1500), (35, 1000, 1501),
+                                   (33, 1025, 900), (64, 2048, 977), (13, 2049, 1220), (6, 257, 5100),
+                                   (28, 2100, 1216), (28, 2100, 1217), (28, 5003, 600), (35, 2100, 400),
+                                   (35, 2100, 410), (64, 3001, 900), (3, 1000, 3500), (6, 300, 12001),
+                                   (64, 999, 2432), (64, 999, 2433), (17, 511, 2432), (17, 513, 2433),
+                                   (14, 100003, 9), (12, 4095, 70),
                                    # clusters that fill the chip, one more and their scratch
                                    (8, 4000, 2304), (8, 4000, 2305), (14, 3000, 2944), (14, 3000, 2945),
                                    (6, 2000, 4736), (6, 2000, 4737), (4, 2000, 9729)])
